@@ -1,6 +1,6 @@
 """Build of the CUDA library libdynot.so (sm_103a) in-tree with nvcc.
 
-Three translation units (the C ABI, the FP32 plan and the FP64 plan) compile
+The C ABI, the plans and the kernels they select compile as separate translation units
 in parallel and link into ``paper_1501_04840_gb300/libdynot.so``.
 """
 from __future__ import annotations
@@ -14,7 +14,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libdynot.so")
-UNITS = ["api", "plan_f32", "plan_f64", "noalloc", "nn", "huepipe"]
+UNITS = (["api", "plan_f32", "plan_f64", "noalloc", "nn", "huepipe"] +
+         ["sel_%s_%s" % (k, t) for k in ("xt", "split", "yc", "mm", "upd") for t in ("f32", "f64")])
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ARCH + ["-O3", "-lineinfo", "-std=c++17", "--expt-relaxed-constexpr", "-Xcompiler", "-fPIC"]
 # extra nvcc flags for tuning experiments (e.g. -DDYNOT_UPD_MINB=2); empty by default

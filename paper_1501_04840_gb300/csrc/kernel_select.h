@@ -1,0 +1,58 @@
+// Kernel selection: which instance of each kernel of an iteration a plan launches.  The functions are defined in
+// kernel_select.cuh and instantiated in the sel_*.cu files, so that the kernels compile as separate units.
+#pragma once
+#include <cuda.h>
+
+#include "hue_kernels.cuh"
+#include "misc_kernels.cuh"
+#include "mm_kernels.cuh"
+#include "rgb_kernels.cuh"
+#include "rgb_update_tma.cuh"
+
+namespace dynot {
+
+constexpr int kThreadsXt = 256;
+constexpr int kThreadsUpd = 128;
+#ifndef DYNOT_YC_W
+#define DYNOT_YC_W 8
+#endif
+constexpr int kW = DYNOT_YC_W;   // x-strip width of the y/colour pass
+
+inline int pmax_for(int P) { return P <= 16 ? 16 : (P <= 32 ? 32 : 64); }
+// lengths with an FFT path: 2^k (64-512) and 3 * 2^k (96 = 16 * 6, 192 = 16 * 12); N1 = fft_n1(n)
+inline bool fft_len(int n) { return n == 64 || n == 96 || n == 128 || n == 192 || n == 256 || n == 512; }
+inline int fft_n1(int n) { return n == 64 ? 8 : (n == 128 ? 8 : 16); }
+// threads per block of the y/colour pass (matches pick_kb)
+// threads of the y/colour pass for strips of W columns: 3 W / 2 row pairs of length n2 per FFT chunk
+// (NT = 12 N1 at W = 8), 256 on the dense path
+constexpr int yc_nt(int m1, int w) { return w == 4 ? 6 * m1 : (w == 8 ? 12 * m1 : 24 * m1); }
+inline int yc_threads(int n2, int w = kW) { return fft_len(n2) ? yc_nt(fft_n1(n2), w) : 256; }
+
+// the folded-product transforms (mm_kernels.cuh): time lengths in register arrays of 16, 24, 32, 48 or 64
+inline int mm_pm(int P) { return P <= 16 ? 16 : (P <= 24 ? 24 : (P <= 32 ? 32 : (P <= 48 ? 48 : 64))); }
+
+template <typename T> using KA = void (*)(Geo<T>, const v4<T>*, const T*, const T*, T*, XtTables, int);
+template <typename T> using KC = void (*)(Geo<T>, const T*, T*, XtTables, int);
+template <typename T> using KB = void (*)(Geo<T>, T*, YcTables, int);
+template <typename T> using KH = void (*)(Geo<T>, T*, HueTables);
+template <typename T> using KRX = void (*)(Geo<T>, const T*, T*, XtTables, int);
+template <typename T> using KCT = void (*)(Geo<T>, T*, const T*);
+template <typename T> using KMF = void (*)(Geo<T>, const v4<T>*, const T*, const T*, T*, MmAxis<T>, const T*);
+template <typename T> using KMI = void (*)(Geo<T>, const T*, T*, MmAxis<T>, const T*);
+template <typename T> using KMY = void (*)(Geo<T>, T*, YcTables, MmAxis<T>, int);
+template <typename T> using KD = void (*)(Geo<T>, Arrays<T>, int, TileLayout, double*);
+using KDT = void (*)(Geo<float>, Arrays<float>, int, double*, int*, const CUtensorMap, const CUtensorMap,
+                     const CUtensorMap);
+
+template <typename T> KA<T> pick_ka(int n, int pm);
+template <typename T> KC<T> pick_kc(int n, int pm);
+template <typename T, bool INV> KRX<T> pick_krx(int n);
+template <typename T> KCT<T> pick_kct(int pm);
+template <typename T> KB<T> pick_kb(int n, int w = kW);
+template <typename T> KMF<T> pick_kmf(int pm);
+template <typename T> KMI<T> pick_kmi(int pm);
+template <typename T> KMY<T> pick_kmy(int C);
+template <typename T> KD<T> pick_kd(int C, bool check, bool wx, bool per_xy);
+KDT pick_kdt(int C, bool check, bool wx);   // FP32, staged by bulk tensor copies
+
+}  // namespace dynot

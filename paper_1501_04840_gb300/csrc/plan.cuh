@@ -16,30 +16,10 @@
 #include <vector>
 
 #include "fft.cuh"
-#include "hue_kernels.cuh"
-#include "misc_kernels.cuh"
+#include "kernel_select.h"
 #include "plan_base.h"
-#include "rgb_kernels.cuh"
-#include "rgb_update_tma.cuh"
 
 namespace dynot {
-
-constexpr int kThreadsXt = 256;
-constexpr int kThreadsUpd = 128;
-#ifndef DYNOT_YC_W
-#define DYNOT_YC_W 8
-#endif
-constexpr int kW = DYNOT_YC_W;   // x-strip width of the y/colour pass
-
-inline int pmax_for(int P) { return P <= 16 ? 16 : (P <= 32 ? 32 : 64); }
-// lengths with an FFT path: 2^k (64-512) and 3 * 2^k (96 = 16 * 6, 192 = 16 * 12); N1 = fft_n1(n)
-inline bool fft_len(int n) { return n == 64 || n == 96 || n == 128 || n == 192 || n == 256 || n == 512; }
-inline int fft_n1(int n) { return n == 64 ? 8 : (n == 128 ? 8 : 16); }
-// threads per block of the y/colour pass (matches pick_kb)
-// threads of the y/colour pass for strips of W columns: 3 W / 2 row pairs of length n2 per FFT chunk
-// (NT = 12 N1 at W = 8), 256 on the dense path
-constexpr int yc_nt(int m1, int w) { return w == 4 ? 6 * m1 : (w == 8 ? 12 * m1 : 24 * m1); }
-inline int yc_threads(int n2, int w = kW) { return fft_len(n2) ? yc_nt(fft_n1(n2), w) : 256; }
 
 inline size_t rnd16(size_t b) { return (b + 15) & ~size_t(15); }
 
@@ -65,122 +45,6 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
-// --------------------------------------------------------------------------
-// kernel selection
-// --------------------------------------------------------------------------
-template <typename T> using KA = void (*)(Geo<T>, const v4<T>*, const T*, const T*, T*, XtTables, int);
-template <typename T> using KC = void (*)(Geo<T>, const T*, T*, XtTables, int);
-template <typename T> using KB = void (*)(Geo<T>, T*, YcTables, int);
-template <typename T> using KH = void (*)(Geo<T>, T*, HueTables);
-
-template <typename T, int PM>
-KA<T> pick_ka_p(int n) {
-  switch (n) {
-    case 64: return k_rhs_fwd_xt<T, 8, 8, PM>;
-    case 96: return k_rhs_fwd_xt<T, 16, 6, PM>;
-    case 128: return k_rhs_fwd_xt<T, 8, 16, PM>;
-    case 192: return k_rhs_fwd_xt<T, 16, 12, PM>;
-    case 256: return k_rhs_fwd_xt<T, 16, 16, PM>;
-    case 512: return k_rhs_fwd_xt<T, 16, 32, PM>;
-    default: return k_rhs_fwd_xt<T, 0, 0, PM>;
-  }
-}
-template <typename T>
-KA<T> pick_ka(int n, int pm) {
-  return pm == 16 ? pick_ka_p<T, 16>(n) : (pm == 32 ? pick_ka_p<T, 32>(n) : pick_ka_p<T, 64>(n));
-}
-template <typename T, int PM>
-KC<T> pick_kc_p(int n) {
-  switch (n) {
-    case 64: return k_inv_xt<T, 8, 8, PM>;
-    case 96: return k_inv_xt<T, 16, 6, PM>;
-    case 128: return k_inv_xt<T, 8, 16, PM>;
-    case 192: return k_inv_xt<T, 16, 12, PM>;
-    case 256: return k_inv_xt<T, 16, 16, PM>;
-    case 512: return k_inv_xt<T, 16, 32, PM>;
-    default: return k_inv_xt<T, 0, 0, PM>;
-  }
-}
-template <typename T>
-KC<T> pick_kc(int n, int pm) {
-  return pm == 16 ? pick_kc_p<T, 16>(n) : (pm == 32 ? pick_kc_p<T, 32>(n) : pick_kc_p<T, 64>(n));
-}
-template <typename T> using KRX = void (*)(Geo<T>, const T*, T*, XtTables, int);
-template <typename T> using KCT = void (*)(Geo<T>, T*, const T*);
-template <typename T, bool INV>
-KRX<T> pick_krx(int n) {
-  switch (n) {
-    case 64: return k_rows_x<T, 8, 8, INV>;
-    case 96: return k_rows_x<T, 16, 6, INV>;
-    case 128: return k_rows_x<T, 8, 16, INV>;
-    case 192: return k_rows_x<T, 16, 12, INV>;
-    case 256: return k_rows_x<T, 16, 16, INV>;
-    case 512: return k_rows_x<T, 16, 32, INV>;
-    default: return k_rows_x<T, 0, 0, INV>;
-  }
-}
-template <typename T>
-KCT<T> pick_kct(int pm) {
-  return pm == 16 ? k_cols_t<T, 16> : (pm == 32 ? k_cols_t<T, 32> : k_cols_t<T, 64>);
-}
-template <typename T, int W>
-KB<T> pick_kb_w(int n) {
-  switch (n) {
-    case 64: return k_solve_yc<T, 8, 8, W, yc_nt(8, W)>;
-    case 96: return k_solve_yc<T, 16, 6, W, yc_nt(16, W)>;
-    case 128: return k_solve_yc<T, 8, 16, W, yc_nt(8, W)>;
-    case 192: return k_solve_yc<T, 16, 12, W, yc_nt(16, W)>;
-    case 256: return k_solve_yc<T, 16, 16, W, yc_nt(16, W)>;
-    case 512: return k_solve_yc<T, 16, 32, W, yc_nt(16, W)>;
-    default: return k_solve_yc<T, 0, 0, kW, 256>;
-  }
-}
-// strips of 4, 8 or 16 columns on the FFT lengths (FP32; the FP64 plan keeps 8)
-template <typename T>
-KB<T> pick_kb(int n, int w = kW) {
-  if constexpr (std::is_same<T, float>::value) {
-    if (fft_len(n) && w == 4) return pick_kb_w<T, 4>(n);
-    if (fft_len(n) && w == 16) return pick_kb_w<T, 16>(n);
-  }
-  return pick_kb_w<T, kW>(n);
-}
-template <typename T> using KD = void (*)(Geo<T>, Arrays<T>, int, TileLayout, double*);
-
-template <typename T, int C, bool PXY>
-KD<T> pick_kd_c(bool check, bool wx) {
-  if (check) return wx ? k_update_tiled<T, C, true, true, PXY> : k_update_tiled<T, C, true, false, PXY>;
-  return wx ? k_update_tiled<T, C, false, true, PXY> : k_update_tiled<T, C, false, false, PXY>;
-}
-template <typename T, bool PXY>
-KD<T> pick_kd_p(int C, bool check, bool wx) {
-  switch (C) {
-    case 1: return pick_kd_c<T, 1, PXY>(check, wx);
-    case 2: return pick_kd_c<T, 2, PXY>(check, wx);
-    case 3: return pick_kd_c<T, 3, PXY>(check, wx);
-    default: return pick_kd_c<T, 4, PXY>(check, wx);
-  }
-}
-template <typename T>
-KD<T> pick_kd(int C, bool check, bool wx, bool per_xy) {
-  return per_xy ? pick_kd_p<T, true>(C, check, wx) : pick_kd_p<T, false>(C, check, wx);
-}
-
-// the update kernel with tensor-memory-accelerator staging (FP32, Neumann x and y)
-using KDT = void (*)(Geo<float>, Arrays<float>, int, double*, int*, const CUtensorMap, const CUtensorMap,
-                     const CUtensorMap);
-template <int C>
-KDT pick_kdt_c(bool check, bool wx) {
-  if (check) return wx ? k_update_tma<C, true, true> : k_update_tma<C, true, false>;
-  return wx ? k_update_tma<C, false, true> : k_update_tma<C, false, false>;
-}
-inline KDT pick_kdt(int C, bool check, bool wx) {
-  switch (C) {
-    case 1: return pick_kdt_c<1>(check, wx);
-    case 2: return pick_kdt_c<2>(check, wx);
-    case 3: return pick_kdt_c<3>(check, wx);
-    default: return pick_kdt_c<4>(check, wx);
-  }
-}
 inline size_t tma_smem(int C) {
   switch (C) {
     case 1: return TmaTiles<1>::total;
@@ -254,6 +118,15 @@ struct Plan final : PlanBase {
   size_t smR = 0, smT = 0;
   KB<T> kb = nullptr;
   KH<T> kh = nullptr;
+  // transforms of axes without an FFT length as folded products
+  bool x_mm = false, y_mm = false;
+  MmAxis<T> mx{}, my{};
+  const T *mtf = nullptr, *mti = nullptr;
+  KMF<T> kmf = nullptr;
+  KMI<T> kmi = nullptr;
+  KMY<T> kmy = nullptr;
+  size_t smMx = 0, smMi = 0, smMy = 0;
+  int ntMf = 0, ntMi = 0, ntMy = 0, wMy = 0;
   bool hue_gemm = false;    // the hue DFTs as dense matrix products (FP32, bins <= kHueGemmMax)
   const T* hwf = nullptr;   // [slot][bin] forward basis
   const T* hwi = nullptr;   // [bin][slot] inverse
@@ -549,6 +422,67 @@ struct Plan final : PlanBase {
   }
   int tune_tc = 0;
 
+  // Axes without an FFT length take the folded products where a (x, t) plane (x) or a strip of columns (y) fits
+  // shared memory and a strip's outputs fit one block's registers; the dense sums keep the rest (axes beyond about
+  // 1500 cells, and planes that the dense passes hold but this layout does not).
+  ot_status choose_mm() {
+    int maxsm = 0;
+    CUDA_OK(cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, device));
+    const char* sx = std::getenv("DYNOT_SPLIT_XT");
+    const bool split = sx && std::strcmp(sx, "1") == 0;
+    auto axis = [](int n, bool per) {
+      MmAxis<T> ax{};
+      ax.n = n;
+      ax.h0 = per ? n / 2 + 1 : (n + 1) / 2;
+      ax.h1 = n - ax.h0;
+      ax.o1 = per;
+      ax.l0 = ax.li = (ax.h0 + 3) / 4 * 4;
+      ax.lf = ax.l0 + (ax.h1 + 3) / 4 * 4;
+      return ax;
+    };
+    mx = axis(n1, g.per1);
+    my = axis(n2, g.per2);
+    const int bufx = mm_buf(mx.l0, mx.lf, mx.li), bufy = mm_buf(my.l0, my.lf, my.li);
+    auto round = [](int n, int lo, int hi) { return std::max(lo, std::min(hi, (n + 31) / 32 * 32)); };
+    if (!x_fft() && !split) {
+      const int pm = mm_pm(P), dense = 4 * n1;
+      const size_t old = xt_layout<T>(nullptr, nullptr, P, n1, pmax, dense, true);
+      smMx = mm_xt_smem<T>(n1, P, pm, bufx, true);
+      smMi = mm_xt_smem<T>(n1, P, pm, bufx, false);
+      // (the kernels' offsets into a problem's a are 32-bit)
+      if ((int)smMx <= maxsm && (int)old <= maxsm && 4 * N < (1ll << 31)) {
+        x_mm = true;
+        kmf = pick_kmf<T>(pm);
+        kmi = pick_kmi<T>(pm);
+        // threads: the columns of the time transform or the products' items, whichever are more
+        const int G = (P + 7) / 8;
+        // threads: the products' items in equal rounds, up to 160 (three or four blocks per SM) where the grid fills the
+        // GPU and as many as have work otherwise
+        const int most = (long long)n2 * C * B > 2 * 152 ? 160 : kMmXtThreads;
+        const int work = G * (mx.lf / 4), rounds = (work + most - 1) / most;
+        ntMf = ntMi = round(std::max((work + rounds - 1) / rounds, std::min(n1, 96)), 64, most);
+      }
+    }
+    if (!y_fft()) {
+      const int wt = mm_yc_wt(C);
+      for (int w = 16; w >= wt; w /= 2) {
+        const int items = mm_yc_items(my.lf, C, w);
+        const size_t sm = mm_yc_smem<T>(n2, C, w, bufy);
+        // narrower strips while the grid has fewer than four blocks per SM (180x135x3x24: 40.0 us with 8 columns, 42.5
+        // with 16; 300x200x3x16: 63.2 against 67.2)
+        const bool more = w > wt && (long long)((n1 + w - 1) / w) * P * B < 4 * 152;
+        if (items > kMmYcThreads || (int)sm > maxsm || more) continue;
+        y_mm = true;
+        wMy = w;
+        smMy = sm;
+        kmy = pick_kmy<T>(C);
+        ntMy = round(items, 128, kMmYcThreads);
+        break;
+      }
+    }
+    return OT_OK;
+  }
+
   // ---- transform tables (computed in double on the host)
   ot_status build_tables() {
     std::vector<char> h;
@@ -591,6 +525,47 @@ struct Plan final : PlanBase {
       }
       return l;
     };
+    // an axis transformed by folded products: its spectrum order [even part][odd part], eigenvalues in that order
+    auto mm_freq = [](int n, bool per, int pos) {   // frequency at a position of the spectrum
+      const int h0 = per ? n / 2 + 1 : (n + 1) / 2;
+      return per ? (pos < h0 ? pos : pos - h0 + 1) : (pos < h0 ? 2 * pos : 2 * (pos - h0) + 1);
+    };
+    auto mm_lam = [&](int n, bool per, double s) {
+      std::vector<double> l(n);
+      for (int q = 0; q < n; ++q) {
+        const double v = std::sin(kPi * mm_freq(n, per, q) / (per ? n : 2.0 * n));
+        l[q] = s * s * 4.0 * v * v;
+      }
+      return l;
+    };
+    auto mm_axis = [&](const MmAxis<T>& ax, size_t (&off)[2]) {
+      const int n = ax.n;
+      const bool per = ax.o1;
+      // basis value of frequency k at sample i: one table of cos(2 pi m / (4 n)) over a full turn
+      std::vector<double> turn(4 * n);
+      for (int m = 0; m < 4 * n; ++m) turn[m] = std::cos(2 * kPi * m / (4.0 * n));
+      auto even = [&](int k, int i) {
+        return per ? turn[(int)((long long)4 * k * i % (4 * n))] : turn[(int)((long long)k * (2 * i + 1) % (4 * n))];
+      };
+      auto odd = [&](int k, int i) { return per ? turn[(int)(((long long)4 * k * i + 3 * n) % (4 * n))] : even(k, i); };
+      std::vector<T> tf((size_t)ax.h0 * ax.lf, T(0)), ti((size_t)ax.h0 * 2 * ax.li, T(0));
+      for (int q = 0; q < ax.h0; ++q) {
+        const int k = mm_freq(n, per, q);
+        const double w = (k == 0 || (per && 2 * k == n)) ? 1.0 / n : 2.0 / n;
+        for (int i = 0; i < ax.h0; ++i) {
+          tf[(size_t)i * ax.lf + q] = (T)even(k, i);
+          ti[(size_t)q * 2 * ax.li + i] = (T)(w * even(k, i));
+        }
+      }
+      for (int q = 0; q < ax.h1; ++q) {
+        const int k = mm_freq(n, per, ax.h0 + q);
+        for (int i = 0; i < ax.h1; ++i) tf[(size_t)i * ax.lf + ax.l0 + q] = (T)odd(k, i + ax.o1);
+        for (int i = 0; i < ax.h0; ++i) ti[(size_t)q * 2 * ax.li + ax.li + i] = (T)(2.0 / n * odd(k, i));
+      }
+      off[0] = put(tf.data(), tf.size() * sizeof(T));
+      off[1] = put(ti.data(), ti.size() * sizeof(T));
+    };
+    size_t o_mx[2] = {}, o_my[2] = {}, o_mtf = 0, o_mti = 0;
     // (cos, sin)(2 pi m / n) pairs, padded to the 4 n values of the cosine table they replace
     auto cs_pad = [&](int n) {
       std::vector<T> c(4 * n, T(0));
@@ -646,9 +621,25 @@ struct Plan final : PlanBase {
       o_hw2 = put(hw.data(), hw.size() * sizeof(T));
       std::vector<T> c2v = g.per2 ? cs_pad(n2) : cos4(n2);
       o_c42 = put(c2v.data(), c2v.size() * sizeof(T));
-      std::vector<double> l1 = g.per1 ? per_lam(n1, grid.axis_scale[0]) : neu_lam(n1, grid.axis_scale[0]);
+      OT_TRY(choose_mm());
+      if (x_mm) {
+        mm_axis(mx, o_mx);
+        const int pm = mm_pm(P), ph = pm / 2, hP = (P + 1) / 2, P4 = (P + 3) / 4 * 4, hP4 = (hP + 3) / 4 * 4;
+        std::vector<T> tf((size_t)P4 * ph, T(0)), ti((size_t)hP4 * pm, T(0));
+        for (int k = 0; k < P; ++k)
+          for (int t = 0; t < P; ++t) {
+            const double c = std::cos(kPi * (double)(k * (2 * t + 1) % (4 * P)) / (2.0 * P));
+            if (t < hP) tf[(size_t)k * ph + t] = (T)c;
+            if (t < hP4) ti[(size_t)t * pm + (k & 1) * ph + k / 2] = (T)((k == 0 ? 1.0 : 2.0) / P * c);
+          }
+        o_mtf = put(tf.data(), tf.size() * sizeof(T));
+        o_mti = put(ti.data(), ti.size() * sizeof(T));
+      }
+      if (y_mm) mm_axis(my, o_my);
       const double s2y = d >= 2 ? grid.axis_scale[1] : 1.0;
-      std::vector<double> l2 = g.per2 ? per_lam(n2, s2y) : neu_lam(n2, s2y);
+      std::vector<double> l1 = x_mm ? mm_lam(n1, g.per1, grid.axis_scale[0])
+                                    : (g.per1 ? per_lam(n1, grid.axis_scale[0]) : neu_lam(n1, grid.axis_scale[0]));
+      std::vector<double> l2 = y_mm ? mm_lam(n2, g.per2, s2y) : (g.per2 ? per_lam(n2, s2y) : neu_lam(n2, s2y));
       std::vector<T> l1T = toT(l1), l2T = toT(l2);
       o_l1 = put(l1T.data(), n1 * sizeof(T));
       o_l1d = put(l1.data(), n1 * sizeof(double));
@@ -749,6 +740,16 @@ struct Plan final : PlanBase {
       yc.lamtd = (const double*)(base + o_ltd);
       yc.Qc = base + o_Q; yc.lamc = base + o_lc; yc.lamcd = (const double*)(base + o_lcd);
       yc.lam_fp64 = thr;
+      auto mm_ptrs = [&](MmAxis<T>& ax, const size_t (&off)[2]) {
+        ax.ft = (const T*)(base + off[0]);
+        ax.it = (const T*)(base + off[1]);
+      };
+      if (x_mm) {
+        mm_ptrs(mx, o_mx);
+        mtf = (const T*)(base + o_mtf);
+        mti = (const T*)(base + o_mti);
+      }
+      if (y_mm) mm_ptrs(my, o_my);
       scrA = x_fft() ? (kThreadsXt / fft_n1(n1)) * n1 : 4 * n1;
       scrB = y_fft() ? (yc_threads(n2, yw) / fft_n1(n2)) * n2 : 4 * n2;
       ka = pick_ka<T>(x_fft() ? n1 : 0, pmax);
@@ -761,7 +762,7 @@ struct Plan final : PlanBase {
       // a (t, x) plane too large for one block's shared memory takes the split x/t passes
       // (DYNOT_SPLIT_XT=1 selects them for any grid, for comparisons)
       const char* sx = std::getenv("DYNOT_SPLIT_XT");
-      split_xt = (int)smA > maxsm || (sx && std::strcmp(sx, "1") == 0);
+      split_xt = !x_mm && ((int)smA > maxsm || (sx && std::strcmp(sx, "1") == 0));
       if (split_xt) {
         scrS = x_fft() ? (256 / fft_n1(n1)) * n1 : (kRowsX * n1 + 1) / 2;
         T *t0p, *t1p;
@@ -786,6 +787,8 @@ struct Plan final : PlanBase {
         CUDA_OK(cudaFuncSetAttribute((const void*)kc, cudaFuncAttributeMaxDynamicSharedMemorySize, maxsm));
       }
       CUDA_OK(cudaFuncSetAttribute((const void*)kb, cudaFuncAttributeMaxDynamicSharedMemorySize, maxsm));
+      for (const void* f : {(const void*)kmf, (const void*)kmi, (const void*)kmy})
+        if (f) CUDA_OK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, maxsm));
     } else {
       if (hue_gemm) {
         CUDA_OK(cudaFuncSetAttribute((const void*)k_hue_tdiv, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -834,7 +837,9 @@ struct Plan final : PlanBase {
   void enqueue_poisson_src(const v4<T>* asrc, cudaEvent_t* evs) {
     if (!hue) {
       if (evs) cudaEventRecord(evs[0], st);
-      if (split_xt) {
+      if (x_mm) {
+        launch_pdl(kmf, dim3(n2, C, B), dim3(ntMf), smMx, st, g, asrc, (const T*)f0n, (const T*)f1n, hat, mx, mtf);
+      } else if (split_xt) {
         k_rhs_cells<T><<<grid1d((long long)B * N), 256, 0, st>>>(g, asrc, (const T*)f0n, (const T*)f1n, hat);
         launch_pdl(krx_f, dim3((P + kRowsX - 1) / kRowsX, n2 * C, B), dim3(256), smR, st, g, (const T*)hat, hat, xt,
                    scrS);
@@ -845,10 +850,15 @@ struct Plan final : PlanBase {
                    scrA);
       }
       if (evs) cudaEventRecord(evs[1], st);
-      launch_pdl(kb, dim3((n1 + yw - 1) / yw, P, B), dim3(yc_threads(y_fft() ? n2 : 0, yw)), smB, st, g, hat, yc,
-                 scrB);
+      if (y_mm)
+        launch_pdl(kmy, dim3((n1 + wMy - 1) / wMy, P, B), dim3(ntMy), smMy, st, g, hat, yc, my, wMy);
+      else
+        launch_pdl(kb, dim3((n1 + yw - 1) / yw, P, B), dim3(yc_threads(y_fft() ? n2 : 0, yw)), smB, st, g, hat, yc,
+                   scrB);
       if (evs) cudaEventRecord(evs[2], st);
-      if (split_xt) {
+      if (x_mm) {
+        launch_pdl(kmi, dim3(n2, C, B), dim3(ntMi), smMi, st, g, (const T*)hat, phi, mx, mti);
+      } else if (split_xt) {
         launch_pdl(kct, dim3((n1 + kColsT - 1) / kColsT, n2 * C, B), dim3(kColsT), smT, st, g, hat,
                    (const T*)xt.Mt_i);
         launch_pdl(krx_i, dim3((P + kRowsX - 1) / kRowsX, n2 * C, B), dim3(256), smR, st, g, (const T*)hat, phi, xt,

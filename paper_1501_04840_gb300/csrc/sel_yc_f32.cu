@@ -1,0 +1,6 @@
+#define SEL_YC
+#include "kernel_select.cuh"
+
+namespace dynot {
+template KB<float> pick_kb<float>(int, int);
+}  // namespace dynot

@@ -1,0 +1,6 @@
+#define SEL_YC
+#include "kernel_select.cuh"
+
+namespace dynot {
+template KB<double> pick_kb<double>(int, int);
+}  // namespace dynot

@@ -1,0 +1,66 @@
+"""GPU parity of the transforms for axis lengths without an FFT (folded products, csrc/mm_kernels.cuh) against the
+FP64 oracle: one projection and one iteration per grid, with the tolerances of test_gpu_parity.  The grids sit at the
+kernels' edges: lengths around whole groups of four outputs and eight time planes, one to four channels, odd and short
+axes, P beside each register width, periodic axes with and without a Nyquist slot, and both precisions."""
+import numpy as np
+import pytest
+
+import oracle as o
+from _helpers import correction_tolerance, f32, oracle_grid, pack_path, random_pair, rel, smooth_field
+
+pytestmark = pytest.mark.gpu
+
+SIG, TAU = 0.3, 0.99 / 0.3
+N, R = "neumann", "periodic"
+RGB = (N, N, R)
+GRIDS = [
+    ((5, 3, 3), RGB, 3),
+    ((37, 61, 4), (N, N, R), 33),
+    ((180, 135, 3), RGB, 24),
+    ((45, 200, 2), (N, N, N), 50),
+    ((321, 33), (N, N), 64),
+    ((63,), (N,), 9),
+    ((31, 17, 3), (R, R, R), 5),
+    ((30, 18, 3), (R, N, R), 25),
+    ((100, 128, 3), RGB, 17),
+    ((128, 100, 1), (N, N, N), 16),
+    ((130, 7, 3), RGB, 49),
+    ((2, 515, 3), RGB, 6),
+]
+IDS = ["x".join(map(str, n)) + "_" + "".join(b[0] for b in bc) + "_P%d" % P for n, bc, P in GRIDS]
+
+
+@pytest.fixture(scope="module")
+def ot():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1501_04840_gb300 import _build
+    _build.build()
+    import paper_1501_04840_gb300 as p
+    p.load_library()
+    return p
+
+
+@pytest.mark.parametrize("precision", [0, 2], ids=["f32", "f64"])
+@pytest.mark.parametrize("n,bc,P", GRIDS, ids=IDS)
+def test_projection(ot, n, bc, P, precision):
+    """Two problems in one plan: phi to 1e-5 (1e-6 in FP64, the float32 output) and x to the FP32 bound of A^T phi."""
+    plan = ot.Plan(ot.grid(n, bc, P, sigma=SIG, tau=TAU, precision=precision), batch=2)
+    g = oracle_grid(n, bc, P)
+    rng = np.random.default_rng(3)
+    ins, refs, phis = [], [], []
+    for s in (4, 5):
+        f0, f1 = random_pair(g, s)
+        am = [smooth_field(g.m_shape(k), rng).astype(np.float32).astype(np.float64) for k in range(g.d)]
+        af = smooth_field(g.f_shape, rng).astype(np.float32).astype(np.float64)
+        m, f, phi = o.project(g, am, af, f0, f1)
+        ins.append((f0, f1, pack_path(g, am, af)))
+        refs.append(pack_path(g, m, f))
+        phis.append(phi)
+    x, phi = plan.project(*(f32(np.stack([p[k] for p in ins])) for k in range(3)), with_phi=True)
+    x, phi = x.reshape(2, -1), phi.reshape(2, -1)
+    for i in range(2):
+        tol = 1e-6 if precision == 2 else 1e-5
+        assert rel(phi[i], phis[i].ravel()) <= tol
+        assert rel(x[i], refs[i]) <= (tol if precision == 2 else correction_tolerance(g, phis[i], refs[i]))
