@@ -65,12 +65,62 @@ __device__ __forceinline__ double cbrt_start(double d) { return cbrt(d); }
 // bounds w <= c + min(d^(1/3), d/c^2) for c > 0 and w <= min(d^(1/3), sqrt(d/|c|))
 // for c <= 0.  q is increasing and convex for z >= max(e, 0), so Newton's
 // method from that bound decreases monotonically to the root.
+__device__ __forceinline__ double rcp_approx(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  return r;
+}
+
+// The root of q(z) = (1 + z)^2 (z - e) - d in FP64 (e + d > 0; |e| and d far from overflow).  The FP64 pipe is a
+// sixty-fourth of the FP32 one, so the start comes from FP32: bound and three Newton steps as prox_J<float> takes
+// them, good to about 1e-7 of |e| + d + z.  From there Newton converges quadratically from either side (q is
+// increasing and convex for z >= max(e, 0), |q''| / (2 q') <= 2): an FP64 step of size s leaves at most 2 s^2 plus
+// what its approximate reciprocal leaves (1e-6 s), so two steps reach rounding and the loop is for starts that
+// cancellation in e + d spoiled.  Update kernel of the FP64 plan at 128x128x3, P = 32: see k_update_tiled.
+__device__ __forceinline__ double prox_root(double e, double d) {
+  const float ef = (float)e, df = (float)d, cf = 1.f + ef;
+  const float cbd = cbrt_start(df);
+  const float zpos = ef + fminf(cbd, fdiv_fast(df, cf * cf));
+  const float zneg = fminf(cbd, sqrt_fast(fdiv_fast(df, fabsf(cf)))) - 1.f;
+  float zf = fmaxf(cf > 0.f ? zpos : zneg, 0.f);
+#pragma unroll
+  for (int it = 0; it < 3; ++it) {
+    const float w = 1.f + zf, zme = zf - ef;
+    zf -= fdiv_fast(w * w * zme - df, w * (2.f * zme + w));
+  }
+  double z = fmax((double)zf, fmax(e, 0.0));   // fmax also drops a NaN of the FP32 start
+  auto newton = [&]() {
+    const double w = 1.0 + z, zme = z - e;
+    const double step = (w * w * zme - d) * rcp_approx(w * (2.0 * zme + w));
+    z -= step;
+    return step;
+  };
+  newton();
+  double step = newton();
+  const double m = fabs(e) + d;
+#pragma unroll 1
+  for (int it = 2; it < 60 && (fabs(step) > 1e-10 * (m + z) || step * step > 1e-16 * (m + z)); ++it) step = newton();
+  return z;
+}
+
 template <typename T>
 __device__ __forceinline__ void prox_J(T am0, T am1, T am2, T af, T sigma, T inv_sigma, T& u0, T& u1, T& u2, T& v) {
   const T s2 = am0 * am0 + am1 * am1 + am2 * am2;
   const T e = sigma * af;
   const T d = T(0.5) * sigma * sigma * s2;
   const bool live = e + d > T(0);
+  if constexpr (sizeof(T) == 8) {
+    // outside this range (and for NaN) the FP64 iteration below
+    if (fabs(e) + d < 1e15) {
+      const T zr = live ? max(prox_root(e, d), T(0)) : T(0);
+      const T rr = zr / (T(1) + zr);
+      u0 = rr * am0;
+      u1 = rr * am1;
+      u2 = rr * am2;
+      v = zr * inv_sigma;
+      return;
+    }
+  }
   const T c = T(1) + e;
   const T cbd = cbrt_start(d);
   // both starts are computed and one is selected, so that the three channels of a cell interleave
