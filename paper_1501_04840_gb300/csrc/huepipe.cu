@@ -194,7 +194,7 @@ __global__ void k_target_hues(int n, int bins, const long long* __restrict__ C, 
 //   k_window_costs  : their sums over the tiles in double, in order; k_argmin_shift takes the least.
 // The costs are the sums of the exhaustive search below term by term, so the shift is the one it finds (rounding
 // moves a minimum of the float sums by a few shifts, the window holds 512 to either side).  n^2 terms become about
-// 1400 n: 0.12 ms in place of 4.7 ms for 65536 pixels.  Hues outside [0, 1] (k_shift_inputs finds them) and images
+// 1400 n: 0.08 ms in place of 4.7 ms for 65536 pixels.  Hues outside [0, 1] (k_shift_inputs finds them) and images
 // of at most kShiftSmall pixels take the exhaustive search, which covers every shift.
 //
 // Exhaustive search and window alike: a block takes
@@ -217,10 +217,11 @@ __device__ __forceinline__ void shift_tile(int n, int s0, int r0, const float* _
     __syncthreads();
     for (int i = tid; i < len; i += kShiftThreads) sx[i] = xs[r0 + i];
     // window entry i holds y at q = r0 - s0 - (kShiftBlock - 1) + i (mod n)
-    const long long qb = (long long)r0 - s0 - (kShiftBlock - 1);
+    int qb = (int)(((long long)r0 - s0 - (kShiftBlock - 1)) % n);
+    if (qb < 0) qb += n;
     for (int i = tid; i < len + kShiftBlock - 1; i += kShiftThreads) {
-      long long q = (qb + i) % n;
-      if (q < 0) q += n;
+      int q = qb + i;
+      while (q >= n) q -= n;
       sy[i] = ys[q];
     }
     __syncthreads();
@@ -298,12 +299,20 @@ __global__ void __launch_bounds__(256) k_shift_slope(int n, int round, const flo
     off += n;
     --turn;
   }
+  // float sums of up to 32 terms, added in double: an error of 1e-7 moves the sign change by n 1e-7 / 2 shifts
   double acc = 0;
+  for (int q0 = threadIdx.x; q0 < n; q0 += 32 * 256) {
+    float part = 0.f;
 #pragma unroll 8
-  for (int q = threadIdx.x; q < n; q += 256) {
-    const int i = q + off;
-    const bool wrap = i >= n;
-    acc += (double)gap[q] * ((double)xs[wrap ? i - n : i] + (wrap ? 1.0 : 0.0));
+    for (int u = 0; u < 32; ++u) {
+      const int q = q0 + 256 * u;
+      if (q < n) {
+        const int i = q + off;
+        const bool wrap = i >= n;
+        part = fmaf(gap[q], xs[wrap ? i - n : i] + (wrap ? 1.f : 0.f), part);
+      }
+    }
+    acc += (double)part;
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
@@ -316,21 +325,21 @@ __global__ void __launch_bounds__(256) k_shift_slope(int n, int round, const flo
     neg[round * kSlopePoints + blockIdx.x] = 2.0 * (sum + (double)turn) - (2.0 * y[n - 1] - 1.0) < 0.0;
   }
 }
-// first shift of the window, in [0, n)
-__device__ __forceinline__ int window_start(int n, const int* __restrict__ neg) {
+// *place: first shift of the window, in [0, n)
+__global__ void __launch_bounds__(kSlopePoints) k_window_place(int n, const int* __restrict__ neg, int* __restrict__ place) {
   long long lo, hi;
   slope_range(n, neg, kSlopeRounds, lo, hi);
   const int s0 = (int)(((lo + hi) / 2 - kShiftBlock / 2) % n);
-  return s0 < 0 ? s0 + n : s0;
+  if (threadIdx.x == 0) *place = s0 < 0 ? s0 + n : s0;
 }
 // one tile of r per block, the kShiftBlock shifts of the window: part[tile][shift]
 __global__ void __launch_bounds__(kShiftThreads) k_shift_window(int n, const float* __restrict__ xs,
                                                                 const float2* __restrict__ ys,
-                                                                const int* __restrict__ neg,
+                                                                const int* __restrict__ place,
                                                                 float* __restrict__ parts) {
   __shared__ float sx[kShiftTile];
   __shared__ float2 sy[kShiftWin];
-  const int s0 = window_start(n, neg);
+  const int s0 = *place;
   float part[kShiftPer];
   shift_tile(n, s0, blockIdx.x * kShiftTile, xs, ys, sx, sy, part);
 #pragma unroll
@@ -338,27 +347,23 @@ __global__ void __launch_bounds__(kShiftThreads) k_shift_window(int n, const flo
     parts[(size_t)blockIdx.x * kShiftBlock + threadIdx.x + kShiftThreads * u] = part[u];
 }
 // cost of the window's shifts, the tiles added in double in the order of the exhaustive search
-__global__ void __launch_bounds__(kSlopePoints) k_window_costs(int n, const int* __restrict__ neg,
-                                                               const int* __restrict__ all,
-                                                               const float* __restrict__ parts,
-                                                               double* __restrict__ cost) {
-  const int s0 = window_start(n, neg);
+__global__ void __launch_bounds__(32) k_window_costs(int n, const int* __restrict__ place, const int* __restrict__ all,
+                                                     const float* __restrict__ parts, double* __restrict__ cost) {
   if (*all) return;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x, tiles = (n + kShiftTile - 1) / kShiftTile;
-  if (i >= kShiftBlock) return;
+  const int i = blockIdx.x * 32 + threadIdx.x, tiles = (n + kShiftTile - 1) / kShiftTile;
   double acc = 0;
-#pragma unroll 16
+#pragma unroll 32
   for (int t = 0; t < tiles; ++t) acc += (double)parts[(size_t)t * kShiftBlock + i];
-  cost[(s0 + i) % n] = acc;
+  cost[(*place + i) % n] = acc;
 }
 
 // the first minimiser of cost (ties to the smaller shift), one block: over all shifts, or over the window
-__global__ void k_argmin_shift(int n, const double* __restrict__ cost, const int* __restrict__ neg,
+__global__ void k_argmin_shift(int n, const double* __restrict__ cost, const int* __restrict__ place,
                                const int* __restrict__ all, int* __restrict__ best) {
   double bc = INFINITY;
   int bs = n;
   const bool every = *all != 0;
-  const int s0 = every ? 0 : window_start(n, neg), cnt = every ? n : kShiftBlock;
+  const int s0 = every ? 0 : *place, cnt = every ? n : kShiftBlock;
   for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
     const int s = (s0 + i) % n;
     const double c = cost[s];
@@ -496,7 +501,7 @@ ot_status ot_hue_specify(int npix, const float* h, int bins, const float* target
                          sizeof(long long) * (bins + 1) + sizeof(float) * npix + sizeof(float2) * npix +
                          sizeof(double) * npix + sizeof(float) * npix +
                          sizeof(float) * kShiftBlock * (size_t)((npix + kShiftTile - 1) / kShiftTile) +
-                         sizeof(int) * (kSlopeRounds * kSlopePoints + 2) + 16 * 12;
+                         sizeof(int) * (kSlopeRounds * kSlopePoints + 3) + 16 * 14;
     CUDA_OK(cudaMalloc(&ws.p, bytes));
     char* q = (char*)ws.p;
     auto take = [&](size_t b) { char* r = q; q += (b + 15) & ~size_t(15); return r; };
@@ -510,6 +515,7 @@ ot_status ot_hue_specify(int npix, const float* h, int bins, const float* target
     double* dcost = (double*)take(sizeof(double) * npix);
     int* dbest = (int*)take(sizeof(int));
     int* dall = (int*)take(sizeof(int));
+    int* dplace = (int*)take(sizeof(int));
     int* dneg = (int*)take(sizeof(int) * kSlopeRounds * kSlopePoints);
     float* dgap = (float*)take(sizeof(float) * npix);
     const int tiles = (npix + kShiftTile - 1) / kShiftTile;
@@ -535,11 +541,12 @@ ot_status ot_hue_specify(int npix, const float* h, int bins, const float* target
     k_shift_inputs<<<grid_for(npix), 256, 0, st>>>(npix, x, y, xs, ys, dgap, dall);
     HP_CHECK();
     for (int k = 0; k < kSlopeRounds; ++k) k_shift_slope<<<kSlopePoints, 256, 0, st>>>(npix, k, xs, dgap, y, dneg);
-    k_shift_window<<<tiles, kShiftThreads, 0, st>>>(npix, xs, ys, dneg, dparts);
-    k_window_costs<<<kShiftBlock / kSlopePoints, kSlopePoints, 0, st>>>(npix, dneg, dall, dparts, dcost);
+    k_window_place<<<1, kSlopePoints, 0, st>>>(npix, dneg, dplace);
+    k_shift_window<<<tiles, kShiftThreads, 0, st>>>(npix, xs, ys, dplace, dparts);
+    k_window_costs<<<kShiftBlock / 32, 32, 0, st>>>(npix, dplace, dall, dparts, dcost);
     k_shift_costs<<<(npix + kShiftBlock - 1) / kShiftBlock, kShiftThreads, 0, st>>>(npix, xs, ys, dall, dcost);
     HP_CHECK();
-    k_argmin_shift<<<1, 1024, 0, st>>>(npix, dcost, dneg, dall, dbest);
+    k_argmin_shift<<<1, 1024, 0, st>>>(npix, dcost, dplace, dall, dbest);
     HP_CHECK();
     k_assign<<<grid_for(npix), 256, 0, st>>>(npix, dbest, idx, y, h_out);
     HP_CHECK();
