@@ -15,6 +15,7 @@
 // The cell update is the shared kernel K_D with n2 = C = 1.
 #pragma once
 #include "common.cuh"
+#include "mm_kernels.cuh"
 #include "rgb_kernels.cuh"
 
 namespace dynot {
@@ -191,285 +192,499 @@ __global__ void __launch_bounds__(256) k_hue_inv(Geo<T> g, const T* __restrict__
 }
 
 // ---------------------------------------------------------------------------
-// The real DFT along the bins as a dense matrix product (FP32 plans with at most kHueGemmMax bins and at
-// least kHueGemmRows rows, where the product fills the GPU; single pairs keep the per-row kernels): the
-// transform of all B P rows at once is C = R W^T with W[slot][i] the basis of the real Fourier slots
-// (forward) or its inverse with the weights 1, 2, ..., 2, (1) / n (inverse, stored transposed).
-//   H_R  hue_rhs  : r = A a - f_b^- per cell (one thread per cell) into a row array;
-//   H_G  gemm_nt  : C[M][N] = sum_k A[m][k] B[n][k], 64 x 64 tiles of 4 x 4 outputs per thread, K in steps
-//                   of 16 through shared memory.
+// The same solve by folded products (mm_kernels.cuh), for bins whose rows fit shared memory:
+//   k_hue_x_fwd : r of a group of time rows and their folded bins in shared memory, then the real DFT, 8 rows x 4
+//                 slots per thread;
+//   k_hue_tt    : the time DCT of SC slot columns, the divide, the inverse DCT;
+//   k_hue_x_inv : the inverse real DFT -> phi, 8 rows x 2 mirrored pairs per thread.
+// SMALL (few rows, a single pair) is bound by latency: blocks of 8 rows x 64 outputs whose table columns are copied
+// while the previous kernel runs, every sum in 16 slices of at most n / 32 steps.  Otherwise the FP32 pipe and the
+// instructions around it bound: 16 rows x all outputs per block, tables in chunks of 8 steps, sums in runs of 16 terms
+// (which keep the rounding error of 16 + n / 32 additions).
 // ---------------------------------------------------------------------------
-constexpr int kHueGemmMax = 1024, kHueGemmRows = 512;
+constexpr int kHueMmThreads = 256;
+constexpr int kHueSlices = 16, kHueItems = 16;   // SMALL: slices of a sum, items (64 table columns) per block
 
+// Rows of X before and after the bins, so that whole steps of 16 stay inside: their table weights are zero.
+__host__ __device__ inline int hue_hpad(int h0) { return (h0 + 15) / 16 * 16; }
+__host__ __device__ inline int hue_xpad(int n, int h0) { return hue_hpad(h0) > n ? hue_hpad(h0) - n : 0; }
+inline size_t hue_mm_vals(int n, int h0, int rb, int items, bool small) {
+  const size_t x = (size_t)(n + 2 * hue_xpad(n, h0)) * (rb + 4);
+  const size_t tab = (size_t)hue_hpad(h0) * 4 * kHueItems, red = (size_t)kHueSlices * 32 * kHueItems;
+  return x + (small ? (tab > red ? tab : red) : (size_t)kMmStages * kMmK * 4 * items);
+}
+
+// Copies of `width` columns of a table (row stride ld) in chunks of 8 rows into slots of row stride ldb.  The place of a
+// thread's first vector and the step between its vectors are found once (a division per vector and chunk took a
+// quarter of the kernel's instructions).
 template <typename T>
-__global__ void __launch_bounds__(256) k_hue_rhs(Geo<T> g, const v4<T>* __restrict__ ap, const T* __restrict__ f0,
-                                                 const T* __restrict__ f1, T* __restrict__ r) {
-  const int n = g.n1, P = g.P;
-  const long long tot = (long long)g.B * P * n;
-  for (long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x; id < tot; id += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(id % n);
-    const long long row = id / n;
-    const int t = (int)(row % P), b = (int)(row / P);
-    if (retired(g, b)) continue;
-    const int im = i > 0 ? i - 1 : n - 1;   // periodic
-    const v4<T> av = ap[id];
-    T v = g.s1 * (av.x - comp<T>(ap, id - i + im, 0));
-    const T fnext = (t == P - 1) ? f1[(size_t)b * n + i] : av.w;
-    const T fprev = (t == 0) ? f0[(size_t)b * n + i] : comp<T>(ap, id - n, 3);
-    v += g.sp * (fnext - fprev);
-    r[id] = v;
+struct HueChunks {
+  const T* tab;
+  T* buf;
+  int ld, ldb, per, r, k, dr, dk, hpad;
+  static constexpr int V = 16 / (int)sizeof(T);
+  __device__ __forceinline__ HueChunks(T* buf_, const T* tab_, int ld_, int width, int ldb_, int hpad_)
+      : tab(tab_), buf(buf_), ld(ld_), ldb(ldb_), per(width / V), hpad(hpad_) {
+    r = threadIdx.x / per;
+    k = threadIdx.x - r * per;
+    dr = blockDim.x / per;
+    dk = blockDim.x - dr * per;
   }
-}
-
-static __global__ void __launch_bounds__(128) k_gemm_nt(int M, int N, int K, const float* __restrict__ A,
-                                                 const float* __restrict__ Bm, float* __restrict__ C) {
-  // 128 threads, 8 x 4 outputs each; K in steps of 32 through two shared-memory buffers: the global loads of
-  // the next step are in flight (in registers) while the products of this one run, one barrier per step
-  constexpr int BK = 32, LD = 68;
-  __shared__ __align__(16) float As[2][BK][LD];
-  __shared__ __align__(16) float Bs[2][BK][LD];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;   // columns 4 tx .. 4 tx + 3, rows 8 ty .. 8 ty + 7
-  const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-  // loads: element q of this thread is row (tid >> 3) + 16 (q >> 2), k (tid & 7) + 8 (q & 3) of the step; a
-  // warp reads 32-byte runs of four rows, and its transposed stores hit 32 different banks
-  const int lk = threadIdx.x & 7, lr = threadIdx.x >> 3;
-  float ra[16], rb[16];
-  auto fetch = [&](int k0) {
-#pragma unroll
-    for (int q = 0; q < 16; ++q) {
-      const int r = lr + 16 * (q >> 2), k = k0 + lk + 8 * (q & 3);
-      ra[q] = (k < K && m0 + r < M) ? A[(size_t)(m0 + r) * K + k] : 0.f;
-      rb[q] = (k < K && n0 + r < N) ? Bm[(size_t)(n0 + r) * K + k] : 0.f;
-    }
-  };
-  auto stash = [&](int buf) {
-#pragma unroll
-    for (int q = 0; q < 16; ++q) {
-      As[buf][lk + 8 * (q & 3)][lr + 16 * (q >> 2)] = ra[q];
-      Bs[buf][lk + 8 * (q & 3)][lr + 16 * (q >> 2)] = rb[q];
-    }
-  };
-  float acc[8][4];
-#pragma unroll
-  for (int i = 0; i < 8; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-  fetch(0);
-  stash(0);
-  __syncthreads();
-  int buf = 0;
-  for (int k0 = 0; k0 < K; k0 += BK) {
-    const bool more = k0 + BK < K;
-    if (more) fetch(k0 + BK);
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      // each run of 16 terms is summed on its own and then added to the total, which keeps the rounding
-      // error of a sum over K terms near that of 16 + K / 16 additions
-      float part[8][4];
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) part[i][j] = 0.f;
-#pragma unroll
-      for (int kk = 0; kk < 16; ++kk) {
-        const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][16 * h + kk][8 * ty]);
-        const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][16 * h + kk][8 * ty + 4]);
-        const float4 b = *reinterpret_cast<const float4*>(&Bs[buf][16 * h + kk][4 * tx]);
-        const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w}, bv[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) part[i][j] = fmaf(av[i], bv[j], part[i][j]);
+  __device__ __forceinline__ void issue(int c) const {
+    if (c * kMmK >= hpad) return;
+    T* dst = buf + (c % kMmStages) * kMmK * ldb;
+    const T* src = tab + (size_t)c * kMmK * ld;
+    for (int i = r, j = k; i < kMmK;) {
+      cp_async16(dst + i * ldb + V * j, src + i * ld + V * j);
+      i += dr;
+      j += dk;
+      if (j >= per) {
+        j -= per;
+        ++i;
       }
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] += part[i][j];
     }
-    if (more) stash(buf ^ 1);   // buffer buf ^ 1 was last read before the previous barrier
-    __syncthreads();
-    buf ^= 1;
   }
+};
+__device__ __forceinline__ void hue_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+// SMALL: `quads` (at most 16) groups of 4 columns of every row
+template <typename T>
+__device__ __forceinline__ void hue_columns(T* buf, const T* tab, int ld, int quads, int ldb, int hpad) {
+  const int k = threadIdx.x % 16;
+  if (k < quads)
+    for (int r = threadIdx.x / 16; r < hpad; r += blockDim.x / 16)
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int m = m0 + 8 * ty + i;
-    if (m >= M) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int nn = n0 + 4 * tx + j;
-      if (nn < N) C[(size_t)m * N + nn] = acc[i][j];
-    }
+      for (int v = 0; v < (int)sizeof(T) / 4; ++v)
+        cp_async16(buf + r * ldb + 4 * k + v * 16 / (int)sizeof(T), tab + (size_t)r * ld + 4 * k + v * 16 / (int)sizeof(T));
+}
+template <typename T>
+__device__ __forceinline__ void hue_zero_pads(T* X, int n, int pad, int ld) {
+  for (int i = threadIdx.x; i < pad * ld; i += blockDim.x) {
+    X[i - pad * ld] = T(0);
+    X[n * ld + i] = T(0);
   }
 }
-
-// C[z][m][n] = sum_k A[m][k] B[z][k][n] for every batch z (A row-major [M][K]; B, C row-major [K][N], [M][N]
-// per batch, batch stride `bs`), the time transforms of all slot columns of the hue rows at once, with the
-// per-step partial sums of k_gemm_nt.  DIV divides every output by its eigenvalue lamt[m] + lam[n] (zero
-// mode -> 0; below lam_fp64 in double), as k_hue_t does between its two products.
-template <bool DIV>
-__global__ void __launch_bounds__(256) k_gemm_tn(int M, int N, int K, const float* __restrict__ A,
-                                                 const float* __restrict__ Bm, float* __restrict__ C, long long bs,
-                                                 HueTables tb) {
-  __shared__ __align__(16) float As[16][68];
-  __shared__ __align__(16) float Bs[16][68];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-  const float* Bz = Bm + (size_t)blockIdx.z * bs;
-  float* Cz = C + (size_t)blockIdx.z * bs;
-  float acc[4][4];
+// visit the cells (row r, bin x) of a rows x n plane, consecutive threads along x; f(index, r, x)
+template <int U, class F>
+__device__ __forceinline__ void hue_cells(int rows, int n, F&& f) {
+  const int nt = blockDim.x, dr = nt / n, dx = nt - dr * n, tot = rows * n;
+  int r = threadIdx.x / n, x = threadIdx.x - r * n;
+  for (int i0 = threadIdx.x; i0 < tot; i0 += U * nt) {
+    int rr[U], xx[U];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-  for (int k0 = 0; k0 < K; k0 += 16) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int idx = threadIdx.x + 256 * q;
-      const int r = idx >> 4, kk = idx & 15;         // A: row r of the tile, k kk
-      As[kk][r] = (m0 + r < M && k0 + kk < K) ? A[(size_t)(m0 + r) * K + k0 + kk] : 0.f;
-      const int kb = idx >> 6, c = idx & 63;         // B: k kb of the tile, column c
-      Bs[kb][c] = (k0 + kb < K && n0 + c < N) ? Bz[(size_t)(k0 + kb) * N + n0 + c] : 0.f;
-    }
-    __syncthreads();
-    float part[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) part[i][j] = 0.f;
-#pragma unroll
-    for (int kk = 0; kk < 16; ++kk) {
-      const float4 a = *reinterpret_cast<const float4*>(&As[kk][4 * ty]);
-      const float4 b = *reinterpret_cast<const float4*>(&Bs[kk][4 * tx]);
-      const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) part[i][j] = fmaf(av[i], bv[j], part[i][j]);
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] += part[i][j];
-    __syncthreads();
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int m = m0 + 4 * ty + i;
-    if (m >= M) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int nn = n0 + 4 * tx + j;
-      if (nn >= N) continue;
-      float v = acc[i][j];
-      if (DIV) {
-        const float lam = ((const float*)tb.lam)[nn] + ((const float*)tb.lamt)[m];
-        if (!(lam > 0.f)) v = 0.f;
-        else if ((double)lam < tb.lam_fp64) v = (float)((double)v / (tb.lamd[nn] + tb.lamtd[m]));
-        else v = v / lam;
+    for (int u = 0; u < U; ++u) {
+      rr[u] = r;
+      xx[u] = x;
+      r += dr;
+      x += dx;
+      if (x >= n) {
+        x -= n;
+        ++r;
       }
-      Cz[(size_t)m * N + nn] = v;
     }
+    f(i0, rr, xx, tot);
   }
 }
 
-// The time transforms of the hue rows with the divide between them, in one launch for P <= 64: block
-// (column block, problem z) takes X = hat[z][0:P][n0:n0+64] into shared memory, forms Y = (Mf X) / lambda
-// there (the forward DCT along t and the eigen-divide of k_gemm_tn<true>) and writes Mi Y back to the same
-// place (k_gemm_tn<false>).  Mf [k][t] and Mi [t][k] are held transposed, so that the four rows of a thread
-// are one 16-byte read; the sums run in the same groups of 16 terms as k_gemm_tn's.
-constexpr int kHueTdivMaxP = 64, kHueTdivLD = 68;
-constexpr size_t kHueTdivSmem = sizeof(float) * 3 * 64 * kHueTdivLD;
-
-static __global__ void __launch_bounds__(256) k_hue_tdiv(int P, int N, const float* __restrict__ Mf,
-                                                  const float* __restrict__ Mi, float* __restrict__ hat,
-                                                  long long bs, HueTables tb) {
-  extern __shared__ __align__(16) float tsm[];
-  constexpr int LD = kHueTdivLD;
-  float* MfT = tsm;              // [t][k]
-  float* MiT = tsm + 64 * LD;    // [k][t]
-  float* X = tsm + 128 * LD;     // [t][n], then Y [k][n]
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int n0 = blockIdx.x * 64;
-  float* hz = hat + (size_t)blockIdx.y * bs;
+template <typename T, bool SMALL>
+__global__ void __launch_bounds__(kHueMmThreads, sizeof(T) == 4 ? 2 : 1)
+    k_hue_x_fwd(Geo<T> g, const v4<T>* __restrict__ ap, const T* __restrict__ f0, const T* __restrict__ f1,
+                T* __restrict__ hat, MmAxis<T> ax, int RB, int QC) {
+  extern __shared__ __align__(16) char smraw[];
+  const int b = blockIdx.z, t0 = blockIdx.x * RB, u0 = blockIdx.y * QC;
+  if (retired(g, b)) return;
+  const int n = g.n1, P = g.P, ld = RB + 4, Q = ax.lf / 4, qn = min(QC, Q - u0), rows = min(RB, P - t0);
+  const int hpad = hue_hpad(ax.h0), pad = hue_xpad(n, ax.h0);
+  T* X = (T*)smraw + pad * ld;
+  T* buf = X + (n + pad) * ld;
+  const T* tab = ax.ft + 4 * u0;
+  const HueChunks<T> chunks(buf, tab, ax.lf, 4 * qn, 4 * QC, hpad);
+  if (SMALL) {
+    hue_columns<T>(buf, tab, ax.lf, qn, 4 * kHueItems, hpad);
+  } else {
+    chunks.issue(0);
+    hue_commit();
+    chunks.issue(1);
+    hue_commit();
+  }
+  hue_zero_pads<T>(X, n, pad, ld);
+  pdl_wait();   // a (previous update) is read from here on
   {
-    // all 48 loads of this thread in flight at once, then the shared-memory stores
-    float vm[16], vi[16], vx[16];
-    const int c = threadIdx.x & 63;
+    constexpr int U = 4;
+    const v4<T>* pc = ap + (size_t)(b * P + t0) * n;
+    const T* as = reinterpret_cast<const T*>(pc);
+    const T *pf0 = f0 + (size_t)b * n, *pf1 = f1 + (size_t)b * n;
+    hue_cells<U>(rows, n, [&](int i0, const int (&rr)[U], const int (&xx)[U], int tot) {
+      v4<T> av[U];
+      T lx[U], lf[U], uf[U];
 #pragma unroll
-    for (int q = 0; q < 16; ++q) {
-      const int r = (threadIdx.x >> 6) + 4 * q;   // row r, column c of the P x P matrices (zero outside)
-      const bool in = r < P && c < P;
-      vm[q] = in ? Mf[(size_t)r * P + c] : 0.f;
-      vi[q] = in ? Mi[(size_t)r * P + c] : 0.f;
-      vx[q] = (r < P && n0 + c < N) ? hz[(size_t)r * N + n0 + c] : 0.f;
-    }
-#pragma unroll
-    for (int q = 0; q < 16; ++q) {
-      const int r = (threadIdx.x >> 6) + 4 * q;
-      MfT[c * LD + r] = vm[q];
-      MiT[c * LD + r] = vi[q];
-      X[r * LD + c] = vx[q];
-    }
-  }
-  __syncthreads();
-  // products of the 4 x 4 outputs of this thread, in runs of 16 terms over the padded 64
-  auto product = [&](const float* AT, float (&acc)[4][4]) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-    for (int k0 = 0; k0 < P; k0 += 16) {
-      float part[4][4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) part[i][j] = 0.f;
-#pragma unroll
-      for (int kk = 0; kk < 16; ++kk) {
-        const float4 a = *reinterpret_cast<const float4*>(&AT[(k0 + kk) * LD + 4 * ty]);
-        const float4 b = *reinterpret_cast<const float4*>(&X[(k0 + kk) * LD + 4 * tx]);
-        const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) part[i][j] = fmaf(av[i], bv[j], part[i][j]);
+      for (int u = 0; u < U; ++u) {
+        const int i = i0 + u * (int)blockDim.x;
+        if (i < tot) {
+          const int t = t0 + rr[u];
+          av[u] = pc[i];
+          lx[u] = as[4 * (xx[u] > 0 ? i - 1 : i + n - 1)];
+          lf[u] = t > 0 ? as[4 * (i - n) + 3] : pf0[xx[u]];
+          uf[u] = t < P - 1 ? av[u].w : pf1[xx[u]];
+        }
       }
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int u = 0; u < U; ++u)
+        if (i0 + u * (int)blockDim.x < tot)
+          X[xx[u] * ld + rr[u]] = g.s1 * (av[u].x - lx[u]) + g.sp * (uf[u] - lf[u]);
+    });
+  }
+  __syncthreads();
+  mm_fold<T>(X, ld, (rows + 3) / 4, ax);
+  T* dst = hat + (size_t)(b * P + t0) * n;
+  if (SMALL) {
+    cp_async_wait_all();
+    __syncthreads();
+    const int ks = threadIdx.x / kHueItems, u = threadIdx.x % kHueItems;
+    const bool odd = 4 * (u0 + u) >= ax.l0;
+    const T* row = X + (odd ? (n - 1 - ks) * ld : ks * ld);
+    const int stride = (odd ? -ld : ld) * kHueSlices;
+    const T* tc = buf + ks * 4 * kHueItems + 4 * u;
+    T acc[32];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] += part[i][j];
+    for (int q = 0; q < 32; ++q) acc[q] = T(0);
+#pragma unroll 4
+    for (int i = 0; i < hpad; i += kHueSlices) {
+      T v[8], m[4];
+      ldv<T, 8>(row, v);
+      ldv<T, 4>(tc, m);
+      row += stride;
+      tc += kHueSlices * 4 * kHueItems;
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[4 * r + e] = fma(v[r], m[e], acc[4 * r + e]);
     }
+    __syncthreads();   // the table's place takes the slices
+#pragma unroll
+    for (int q = 0; q < 32; ++q) buf[(ks * 32 + q) * kHueItems + u] = acc[q];
+    __syncthreads();
+    pdl_trigger();
+    for (int o = threadIdx.x; o < 8 * 4 * kHueItems; o += blockDim.x) {
+      const int e = o & 3, uo = (o >> 2) % kHueItems, r = o / (4 * kHueItems);
+      const bool od = 4 * (u0 + uo) >= ax.l0;
+      const int q = 4 * (u0 + uo) - (od ? ax.l0 : 0) + e;
+      if (uo >= qn || r >= rows || q >= (od ? ax.h1 : ax.h0)) continue;
+      T sum = T(0);
+#pragma unroll
+      for (int k = 0; k < kHueSlices; ++k) sum += buf[(k * 32 + 4 * r + e) * kHueItems + uo];
+      dst[(size_t)r * n + (od ? ax.h0 : 0) + q] = sum;
+    }
+    return;
+  }
+  const int rg = threadIdx.x / QC, u = threadIdx.x - rg * QC;
+  const bool live = u < qn && 8 * rg < rows;
+  const bool odd = 4 * (u0 + u) >= ax.l0;
+  const int stride = odd ? -ld : ld;
+  const T* row = X + (odd ? (n - 1) * ld : 0) + 8 * rg;
+  T acc[8][4], part[8][4];
+  mm_zero<T>(acc);
+  mm_zero<T>(part);
+#pragma unroll 1
+  for (int c = 0; c * kMmK < hpad; ++c) {
+    asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+    __syncthreads();   // chunk c is there (and, at first, the folded rows), and every thread is done with chunk c - 1
+    chunks.issue(c + 2);
+    hue_commit();
+    if (!live) continue;
+    const T* tc = buf + (c % kMmStages) * kMmK * 4 * QC + 4 * u;
+#pragma unroll
+    for (int j = 0; j < kMmK; ++j) {
+      T v[8], m[4];
+      ldv<T, 8>(row, v);
+      ldv<T, 4>(tc, m);
+      row += stride;
+      tc += 4 * QC;
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) part[r][e] = fma(v[r], m[e], part[r][e]);
+    }
+    if (c & 1) {
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          acc[r][e] += part[r][e];
+          part[r][e] = T(0);
+        }
+    }
+  }
+  pdl_trigger();
+  if (!live) return;
+  const int q0 = 4 * (u0 + u) - (odd ? ax.l0 : 0), h = odd ? ax.h1 : ax.h0;
+  dst += (size_t)(8 * rg) * n + (odd ? ax.h0 : 0) + q0;
+#pragma unroll
+  for (int r = 0; r < 8; ++r)
+    if (8 * rg + r < rows) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (q0 + e < h) dst[(size_t)r * n + e] = acc[r][e];
+    }
+}
+
+template <typename T, bool SMALL>
+__global__ void __launch_bounds__(kHueMmThreads, sizeof(T) == 4 ? 2 : 1)
+    k_hue_x_inv(Geo<T> g, const T* __restrict__ hat, T* __restrict__ phi, MmAxis<T> ax, int RB, int IC) {
+  extern __shared__ __align__(16) char smraw[];
+  const int b = blockIdx.z, t0 = blockIdx.x * RB, i00 = 2 * blockIdx.y * IC;   // IC even: table columns in whole vectors
+  if (retired(g, b)) return;
+  const int n = g.n1, P = g.P, ld = RB + 4, rows = min(RB, P - t0), wid = min(2 * IC, ax.li - i00);
+  const int hpad = hue_hpad(ax.h0), pad = hue_xpad(n, ax.h0);
+  T* X = (T*)smraw + pad * ld;   // [slot][t]
+  T* buf = X + (n + pad) * ld;
+  const HueChunks<T> ce(buf, ax.it + i00, 2 * ax.li, wid, 4 * IC, hpad);
+  const HueChunks<T> co(buf + 2 * IC, ax.it + ax.li + i00, 2 * ax.li, wid, 4 * IC, hpad);
+  auto issue = [&](int c) {
+    ce.issue(c);
+    co.issue(c);
+    hue_commit();
   };
-  float acc[4][4];
-  product(MfT, acc);
-  __syncthreads();   // every thread is done with X: it now takes Y
+  if (SMALL) {
+    hue_columns<T>(buf, ax.it + i00, 2 * ax.li, wid / 4, 4 * kHueItems, hpad);
+    hue_columns<T>(buf + 2 * kHueItems, ax.it + ax.li + i00, 2 * ax.li, wid / 4, 4 * kHueItems, hpad);
+  } else {
+    issue(0);
+    issue(1);
+  }
+  hue_zero_pads<T>(X, n, pad, ld);
+  pdl_wait();   // the spectral array (time transforms) is read from here on
+  {
+    constexpr int U = 8;
+    const T* src = hat + (size_t)(b * P + t0) * n;
+    hue_cells<U>(rows, n, [&](int i0, const int (&rr)[U], const int (&xx)[U], int tot) {
+      T v[U];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int m = 4 * ty + i;
+      for (int u = 0; u < U; ++u)
+        if (i0 + u * (int)blockDim.x < tot) v[u] = src[i0 + u * (int)blockDim.x];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int nn = n0 + 4 * tx + j;
-      float v = 0.f;
-      if (m < P && nn < N) {
-        v = acc[i][j];
-        const float lam = ((const float*)tb.lam)[nn] + ((const float*)tb.lamt)[m];
-        if (!(lam > 0.f)) v = 0.f;
-        else if ((double)lam < tb.lam_fp64) v = (float)((double)v / (tb.lamd[nn] + tb.lamtd[m]));
-        else v = v / lam;
+      for (int u = 0; u < U; ++u)
+        if (i0 + u * (int)blockDim.x < tot) X[xx[u] * ld + rr[u]] = v[u];
+    });
+  }
+  T* dst = phi + (size_t)(b * P + t0) * n;
+  // the steps past the odd part's rows read the pads or the even part's rows of other steps: zero weights
+  const int oddlast = n + pad - 1;
+  if (SMALL) {
+    cp_async_wait_all();
+    __syncthreads();
+    const int ks = threadIdx.x / kHueItems, u = threadIdx.x % kHueItems;
+    const T* tc = buf + ks * 4 * kHueItems + 2 * u;
+    T acc[32];   // E and O of the pair's two samples: acc[4 r + 2 part + e]
+#pragma unroll
+    for (int q = 0; q < 32; ++q) acc[q] = T(0);
+#pragma unroll 2
+    for (int q = ks; q < hpad; q += kHueSlices) {
+      T v[8], w[8], m[2], k[2];
+      ldv<T, 8>(X + q * ld, v);
+      ldv<T, 8>(X + min(ax.h0 + q, oddlast) * ld, w);
+      ldv<T, 2>(tc, m);
+      ldv<T, 2>(tc + 2 * kHueItems, k);
+      tc += kHueSlices * 4 * kHueItems;
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          acc[4 * r + e] = fma(v[r], m[e], acc[4 * r + e]);
+          acc[4 * r + 2 + e] = fma(w[r], k[e], acc[4 * r + 2 + e]);
+        }
+    }
+    __syncthreads();   // the table's place takes the slices
+#pragma unroll
+    for (int q = 0; q < 32; ++q) buf[(ks * 32 + q) * kHueItems + u] = acc[q];
+    __syncthreads();
+    pdl_trigger();
+    for (int o = threadIdx.x; o < 8 * 2 * kHueItems; o += blockDim.x) {
+      const int e = o & 1, uo = (o >> 1) % kHueItems, r = o / (2 * kHueItems), i = i00 + 2 * uo + e;
+      if (i >= ax.h0 || r >= rows) continue;
+      T E = T(0), O = T(0);
+#pragma unroll
+      for (int k = 0; k < kHueSlices; ++k) {
+        E += buf[(k * 32 + 4 * r + e) * kHueItems + uo];
+        O += buf[(k * 32 + 4 * r + 2 + e) * kHueItems + uo];
       }
-      X[m * LD + 4 * tx + j] = v;
+      const int mi = ax.mirror(i);
+      dst[(size_t)r * n + i] = E + O;
+      if (mi != i) dst[(size_t)r * n + mi] = E - O;
+    }
+    return;
+  }
+  const int rg = threadIdx.x / IC, u = threadIdx.x - rg * IC, i0 = i00 + 2 * u;
+  const bool live = i0 < ax.h0 && 8 * rg < rows;
+  const T* even = X + 8 * rg;
+  T acc[8][4], part[8][4];   // E and O of the pair's two samples: [r][2 part + e]
+  mm_zero<T>(acc);
+  mm_zero<T>(part);
+#pragma unroll 1
+  for (int c = 0; c * kMmK < hpad; ++c) {
+    asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+    __syncthreads();
+    issue(c + 2);
+    if (!live) continue;
+    const T* tc = buf + (c % kMmStages) * kMmK * 4 * IC + 2 * u;
+#pragma unroll
+    for (int j = 0; j < kMmK; ++j) {
+      const int q = c * kMmK + j;
+      T v[8], m[2];
+      ldv<T, 8>(even + q * ld, v);
+      ldv<T, 2>(tc, m);
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) part[r][e] = fma(v[r], m[e], part[r][e]);
+      ldv<T, 8>(even + min(ax.h0 + q, oddlast) * ld, v);
+      ldv<T, 2>(tc + 2 * IC, m);
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) part[r][2 + e] = fma(v[r], m[e], part[r][2 + e]);
+      tc += 4 * IC;
+    }
+    if (c & 1) {
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          acc[r][e] += part[r][e];
+          part[r][e] = T(0);
+        }
+    }
+  }
+  pdl_trigger();
+  if (!live) return;
+  dst += (size_t)(8 * rg) * n;
+#pragma unroll
+  for (int e = 0; e < 2; ++e) {
+    const int i = i0 + e;
+    if (i >= ax.h0) continue;
+    const int mi = ax.mirror(i);
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+      if (8 * rg + r < rows) {
+        dst[(size_t)r * n + i] = acc[r][e] + acc[r][2 + e];
+        if (mi != i) dst[(size_t)r * n + mi] = acc[r][e] - acc[r][2 + e];
+      }
+  }
+}
+
+// Tables of k_hue_tt: tf [t < hP][P4] forward, te / to [j][h4] inverse weights of frequencies 2 j and 2 j + 1 at the
+// samples t < hP; P4, h4 = P and hP = (P + 1) / 2 rounded up to whole vectors of 4, absent entries zero.
+__host__ __device__ inline int hue_p4(int P) { return (P + 3) / 4 * 4; }
+__host__ __device__ inline int hue_h4(int P) { return ((P + 1) / 2 + 3) / 4 * 4; }
+inline size_t hue_tt_vals(int P, int SC) {
+  const int hP = (P + 1) / 2;
+  return (size_t)hP * hue_p4(P) + 2 * (size_t)hP * hue_h4(P) + 2 * (size_t)(hue_p4(P) + 2) * SC;
+}
+// SMALL: 8 slots per block, one slot and 2 frequencies (then 1 mirrored pair of samples) per thread; otherwise 32
+// slots, 2 slots and 4 frequencies (2 pairs) per thread
+template <bool SMALL> struct HueTt {
+  static constexpr int SC = SMALL ? 8 : 32, ST = SMALL ? 1 : 2, KT = SMALL ? 2 : 4, TT = SMALL ? 1 : 2, LANES = SC / ST;
+};
+template <typename T, bool SMALL>
+__global__ void __launch_bounds__(256) k_hue_tt(Geo<T> g, T* __restrict__ hat, HueTables tb, const T* __restrict__ tabs) {
+  using L = HueTt<SMALL>;
+  constexpr int SC = L::SC, ST = L::ST, KT = L::KT, TT = L::TT;
+  extern __shared__ __align__(16) char smraw[];
+  const int b = blockIdx.y, x0 = blockIdx.x * SC;
+  if (retired(g, b)) return;
+  const int n = g.n1, P = g.P, hP = (P + 1) / 2, P4 = hue_p4(P), h4 = hue_h4(P), act = min(SC, n - x0);
+  T* tf = (T*)smraw;
+  T* te = tf + hP * P4;
+  T* to = te + hP * h4;
+  T* V = to + hP * h4;       // [t][slot]: samples, then sums (t < hP) and differences (mirrored rows)
+  T* Y = V + (P4 + 2) * SC;  // [k][slot], two rows more
+  {
+    constexpr int W = 16 / (int)sizeof(T);
+    const int cnt = hP * P4 + 2 * hP * h4;
+    for (int i = W * threadIdx.x; i < cnt; i += W * blockDim.x) cp_async16(tf + i, tabs + i);
+  }
+  for (int i = threadIdx.x; i < 2 * SC; i += blockDim.x) Y[P * SC + i] = T(0);   // read with zero weights
+  const int xs = threadIdx.x % L::LANES * ST, lane0 = threadIdx.x / L::LANES, lanes = blockDim.x / L::LANES;
+  pdl_wait();   // the spectral array (bin transform) is read from here on
+  T* base = hat + (size_t)b * P * n + x0;
+  {
+    // mirrored samples folded on the way in
+    const int x = threadIdx.x % SC;
+#pragma unroll 4
+    for (int t = threadIdx.x / SC; t < hP; t += blockDim.x / SC) {
+      const T lo = x < act ? base[(size_t)t * n + x] : T(0), hi = x < act ? base[(size_t)(P - 1 - t) * n + x] : T(0);
+      const bool mid = 2 * t == P - 1;
+      V[(P - 1 - t) * SC + x] = mid ? lo : lo - hi;
+      if (!mid) V[t * SC + x] = lo + hi;
+    }
+  }
+  cp_async_wait_all();
+  __syncthreads();
+  for (int k0 = KT * lane0; k0 < P; k0 += KT * lanes) {
+    T acc[KT][ST];
+    mm_zero<T, KT, ST>(acc);
+    const T *ps = V + xs, *pd = V + (P - 1) * SC + xs, *pm = tf + k0;
+#pragma unroll 8
+    for (int t = 0; t < hP; ++t) {
+      T m[KT];
+      ldv<T, KT>(pm, m);
+#pragma unroll
+      for (int q = 0; q < ST; ++q) {
+        const T s = ps[q], d = pd[q];   // the middle row of odd P meets zero weights of the odd frequencies
+#pragma unroll
+        for (int e = 0; e < KT; ++e) acc[e][q] = fma(m[e], e & 1 ? d : s, acc[e][q]);
+      }
+      ps += SC;
+      pd -= SC;
+      pm += P4;
+    }
+#pragma unroll
+    for (int e = 0; e < KT; ++e) {
+      const int k = k0 + e;
+      if (k >= P) continue;
+#pragma unroll
+      for (int q = 0; q < ST; ++q) {
+        const int slot = min(x0 + xs + q, n - 1);
+        T v = acc[e][q];
+        const T lam = ((const T*)tb.lam)[slot] + ((const T*)tb.lamt)[k];
+        if (!(lam > T(0))) v = T(0);
+        else if ((double)lam < tb.lam_fp64) v = (T)((double)v / (tb.lamd[slot] + tb.lamtd[k]));
+        else v = v / lam;
+        Y[k * SC + xs + q] = v;
+      }
     }
   }
   __syncthreads();
-  product(MiT, acc);
+  pdl_trigger();
+  for (int t0 = TT * lane0; t0 < hP; t0 += TT * lanes) {
+    T E[TT][ST], O[TT][ST];
+    mm_zero<T, TT, ST>(E);
+    mm_zero<T, TT, ST>(O);
+    const T *py = Y + xs, *pe = te + t0, *po = to + t0;
+#pragma unroll 8
+    for (int j = 0; j < hP; ++j) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int t = 4 * ty + i;
-    if (t >= P) continue;
+      for (int q = 0; q < ST; ++q) {
+        const T a = py[q], c = py[SC + q];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int nn = n0 + 4 * tx + j;
-      if (nn < N) hz[(size_t)t * N + nn] = acc[i][j];
+        for (int e = 0; e < TT; ++e) {
+          E[e][q] = fma(pe[e], a, E[e][q]);
+          O[e][q] = fma(po[e], c, O[e][q]);
+        }
+      }
+      py += 2 * SC;
+      pe += h4;
+      po += h4;
+    }
+#pragma unroll
+    for (int e = 0; e < TT; ++e) {
+      const int t = t0 + e;
+      if (t >= hP) continue;
+#pragma unroll
+      for (int q = 0; q < ST; ++q)
+        if (xs + q < act) {
+          base[(size_t)t * n + xs + q] = E[e][q] + O[e][q];
+          if (t != P - 1 - t) base[(size_t)(P - 1 - t) * n + xs + q] = E[e][q] - O[e][q];
+        }
     }
   }
 }

@@ -127,11 +127,16 @@ struct Plan final : PlanBase {
   KMY<T> kmy = nullptr;
   size_t smMx = 0, smMi = 0, smMy = 0;
   int ntMf = 0, ntMi = 0, ntMy = 0, wMy = 0;
-  bool hue_gemm = false;    // the hue DFTs as dense matrix products (FP32, bins <= kHueGemmMax)
-  const T* hwf = nullptr;   // [slot][bin] forward basis
-  const T* hwi = nullptr;   // [bin][slot] inverse
-  const T* hmf = nullptr;   // [k][t] forward DCT along t (P x P)
-  const T* hmi = nullptr;   // [t][k] its inverse
+  // hue transforms as folded products (hue_kernels.cuh); mx holds the bins' tables
+  struct HueLaunch {
+    int rb = 8, chunk = 0, nch = 1, nt = 0;
+    size_t smem = 0;
+  };
+  bool hue_mm = false, hue_small = false;
+  HueLaunch hf, hi;
+  int hsc = 32;
+  size_t smTt = 0;
+  const T* htt = nullptr;   // tables of k_hue_tt
   bool tiled = false;       // tiled update kernel (up to four colour channels)
   bool use_tma = false;     // the tiled update stages its planes with bulk tensor copies
   CUtensorMap tmA[2]{}, tmB[2]{}, tmP{};   // a[p], b[p] and phi for k_update_tma
@@ -422,6 +427,49 @@ struct Plan final : PlanBase {
   }
   int tune_tc = 0;
 
+  static MmAxis<T> mm_shape(int n, bool per) {
+    MmAxis<T> ax{};
+    ax.n = n;
+    ax.h0 = per ? n / 2 + 1 : (n + 1) / 2;
+    ax.h1 = n - ax.h0;
+    ax.o1 = per;
+    ax.l0 = ax.li = (ax.h0 + 3) / 4 * 4;
+    ax.lf = ax.l0 + (ax.h1 + 3) / 4 * 4;
+    return ax;
+  }
+
+  // The hue transforms as folded products, where the rows fit shared memory (3000 bins do).  Fewer row groups than
+  // SMs (a single pair): the latency-bound form of the kernels, where its table columns fit.
+  ot_status choose_hue_mm() {
+    int maxsm = 0;
+    CUDA_OK(cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, device));
+    mx = mm_shape(n1, true);
+    const int items_f = mx.lf / 4, items_i = (mx.h0 + 1) / 2;   // outputs per 8 rows, 4 table columns each
+    auto pick = [&](int items, int even) {
+      HueLaunch h;
+      h.rb = !hue_small && P > 8 ? 16 : 8;
+      if (hue_small) {
+        h.chunk = kHueItems;
+        h.nt = kHueMmThreads;
+      } else {
+        const int cap = kHueMmThreads / (h.rb / 8), nch = (items + cap - 1) / cap;
+        h.chunk = ((items + nch - 1) / nch + even - 1) / even * even;
+        h.nt = std::max(128, (h.rb / 8 * h.chunk + 31) / 32 * 32);
+      }
+      h.nch = (items + h.chunk - 1) / h.chunk;
+      h.smem = sizeof(T) * hue_mm_vals(n1, mx.h0, h.rb, h.chunk, hue_small);
+      return h;
+    };
+    const long long G8 = (long long)((P + 7) / 8) * B;
+    hue_small = G8 < 152 && (int)(sizeof(T) * hue_mm_vals(n1, mx.h0, 8, kHueItems, true)) <= maxsm;
+    hf = pick(items_f, 1);
+    hi = pick(items_i, 2);
+    hsc = hue_small ? HueTt<true>::SC : HueTt<false>::SC;
+    smTt = sizeof(T) * hue_tt_vals(P, hsc);
+    hue_mm = (int)std::max(std::max(hf.smem, hi.smem), smTt) <= maxsm && hf.nt <= kHueMmThreads && hi.nt <= kHueMmThreads;
+    return OT_OK;
+  }
+
   // Axes without an FFT length take the folded products where a (x, t) plane (x) or a strip of columns (y) fits
   // shared memory and a strip's outputs fit one block's registers; the dense sums keep the rest (axes beyond about
   // 1500 cells, and planes that the dense passes hold but this layout does not).
@@ -430,18 +478,8 @@ struct Plan final : PlanBase {
     CUDA_OK(cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, device));
     const char* sx = std::getenv("DYNOT_SPLIT_XT");
     const bool split = sx && std::strcmp(sx, "1") == 0;
-    auto axis = [](int n, bool per) {
-      MmAxis<T> ax{};
-      ax.n = n;
-      ax.h0 = per ? n / 2 + 1 : (n + 1) / 2;
-      ax.h1 = n - ax.h0;
-      ax.o1 = per;
-      ax.l0 = ax.li = (ax.h0 + 3) / 4 * 4;
-      ax.lf = ax.l0 + (ax.h1 + 3) / 4 * 4;
-      return ax;
-    };
-    mx = axis(n1, g.per1);
-    my = axis(n2, g.per2);
+    mx = mm_shape(n1, g.per1);
+    my = mm_shape(n2, g.per2);
     const int bufx = mm_buf(mx.l0, mx.lf, mx.li), bufy = mm_buf(my.l0, my.lf, my.li);
     auto round = [](int n, int lo, int hi) { return std::max(lo, std::min(hi, (n + 31) / 32 * 32)); };
     if (!x_fft() && !split) {
@@ -541,26 +579,46 @@ struct Plan final : PlanBase {
     auto mm_axis = [&](const MmAxis<T>& ax, size_t (&off)[2]) {
       const int n = ax.n;
       const bool per = ax.o1;
-      // basis value of frequency k at sample i: one table of cos(2 pi m / (4 n)) over a full turn
-      std::vector<double> turn(4 * n);
-      for (int m = 0; m < 4 * n; ++m) turn[m] = std::cos(2 * kPi * m / (4.0 * n));
-      auto even = [&](int k, int i) {
-        return per ? turn[(int)((long long)4 * k * i % (4 * n))] : turn[(int)((long long)k * (2 * i + 1) % (4 * n))];
+      // cos(2 pi m / (4 n)) over a full turn (sin: m + 3 n); along a table row the index m advances by a constant
+      std::vector<T> turn(4 * n), turn2(4 * n);
+      for (int m = 0; m < 4 * n; ++m) {
+        const double v = std::cos(2 * kPi * m / (4.0 * n));
+        turn[m] = (T)v;
+        turn2[m] = (T)(2.0 / n * v);
+      }
+      auto fill = [&](T* dst, int cnt, const std::vector<T>& tab, long long m0, long long step) {
+        int m = (int)(m0 % (4 * n)), d = (int)(step % (4 * n));
+        for (int i = 0; i < cnt; ++i) {
+          dst[i] = tab[m];
+          m += d;
+          if (m >= 4 * n) m -= 4 * n;
+        }
       };
-      auto odd = [&](int k, int i) { return per ? turn[(int)(((long long)4 * k * i + 3 * n) % (4 * n))] : even(k, i); };
-      std::vector<T> tf((size_t)ax.h0 * ax.lf, T(0)), ti((size_t)ax.h0 * 2 * ax.li, T(0));
-      for (int q = 0; q < ax.h0; ++q) {
-        const int k = mm_freq(n, per, q);
-        const double w = (k == 0 || (per && 2 * k == n)) ? 1.0 / n : 2.0 / n;
-        for (int i = 0; i < ax.h0; ++i) {
-          tf[(size_t)i * ax.lf + q] = (T)even(k, i);
-          ti[(size_t)q * 2 * ax.li + i] = (T)(w * even(k, i));
+      const size_t rows = hue_hpad(ax.h0);   // zero rows up to whole groups of 16 (read by the hue kernels)
+      std::vector<T> tf(rows * ax.lf, T(0)), ti(rows * 2 * ax.li, T(0));
+      for (int i = 0; i < ax.h0; ++i) {
+        T* row = tf.data() + (size_t)i * ax.lf;
+        if (per) {   // cos(2 pi q i / n); sin(2 pi (q + 1) (i + 1) / n)
+          fill(row, ax.h0, turn, 0, 4ll * i);
+          if (i < ax.h1) fill(row + ax.l0, ax.h1, turn, 4ll * (i + 1) + 3ll * n, 4ll * (i + 1));
+        } else {     // cos(pi k (2 i + 1) / (2 n)) for k = 2 q and 2 q + 1
+          fill(row, ax.h0, turn, 0, 2ll * (2 * i + 1));
+          if (i < ax.h1) fill(row + ax.l0, ax.h1, turn, 2 * i + 1, 2ll * (2 * i + 1));
         }
       }
-      for (int q = 0; q < ax.h1; ++q) {
-        const int k = mm_freq(n, per, ax.h0 + q);
-        for (int i = 0; i < ax.h1; ++i) tf[(size_t)i * ax.lf + ax.l0 + q] = (T)odd(k, i + ax.o1);
-        for (int i = 0; i < ax.h0; ++i) ti[(size_t)q * 2 * ax.li + ax.li + i] = (T)(2.0 / n * odd(k, i));
+      for (int q = 0; q < ax.h0; ++q) {
+        T* row = ti.data() + (size_t)q * 2 * ax.li;
+        const int k = mm_freq(n, per, q);
+        const bool one = k == 0 || (per && 2 * k == n);   // weight 1 / n, all others 2 / n
+        if (per) {
+          fill(row, ax.h0, turn2, 0, 4ll * q);
+          if (q < ax.h1) fill(row + ax.li, ax.h0, turn2, 3ll * n, 4ll * (q + 1));
+        } else {
+          fill(row, ax.h0, turn2, k, 2ll * k);
+          if (q < ax.h1) fill(row + ax.li, ax.h0, turn2, k + 1, 2ll * (k + 1));
+        }
+        if (one)
+          for (int i = 0; i < ax.h0; ++i) row[i] *= T(0.5);
       }
       off[0] = put(tf.data(), tf.size() * sizeof(T));
       off[1] = put(ti.data(), ti.size() * sizeof(T));
@@ -607,8 +665,7 @@ struct Plan final : PlanBase {
     size_t o_ltd = put(lt.data(), P * sizeof(double));
 
     size_t o_tw1 = 0, o_hw1 = 0, o_c41 = 0, o_tw2 = 0, o_hw2 = 0, o_c42 = 0, o_l1 = 0, o_l1d = 0, o_l2 = 0,
-           o_l2d = 0, o_Q = 0, o_lc = 0, o_lcd = 0, o_cs = 0, o_hl = 0, o_hld = 0, o_wf = 0, o_wi = 0, o_mf = 0,
-           o_mi = 0;
+           o_l2d = 0, o_Q = 0, o_lc = 0, o_lcd = 0, o_cs = 0, o_hl = 0, o_hld = 0, o_tt = 0;
     if (!hue) {
       std::vector<T> tw, hw;
       twid(n1, tw, hw);
@@ -677,55 +734,30 @@ struct Plan final : PlanBase {
     } else {
       const int n = n1;
       std::vector<T> cs(2 * n);
+      OT_TRY(choose_hue_mm());
+      if (hue_mm) {
+        mm_axis(mx, o_mx);
+        const int hP = (P + 1) / 2, P4 = hue_p4(P), h4 = hue_h4(P);
+        std::vector<T> tt((size_t)hP * P4 + 2 * (size_t)hP * h4, T(0));
+        T *te = tt.data() + (size_t)hP * P4, *to = te + (size_t)hP * h4;
+        for (int k = 0; k < P; ++k)
+          for (int t = 0; t < hP; ++t) {
+            const double c = std::cos(kPi * (double)(k * (2 * t + 1) % (4 * P)) / (2.0 * P));
+            tt[(size_t)t * P4 + k] = (T)c;
+            (k & 1 ? to : te)[(size_t)(k / 2) * h4 + t] = (T)((k == 0 ? 1.0 : 2.0) / P * c);
+          }
+        o_tt = put(tt.data(), tt.size() * sizeof(T));
+      }
       std::vector<double> hl(n);
       for (int m = 0; m < n; ++m) {
         cs[2 * m] = (T)std::cos(2 * kPi * m / n);
         cs[2 * m + 1] = (T)std::sin(2 * kPi * m / n);
       }
-      const double s1 = grid.axis_scale[0];
-      for (int slot = 0; slot < n; ++slot) {
-        int j = (slot + 1) / 2;
-        if (n % 2 == 0 && slot == n - 1) j = n / 2;
-        const double v = std::sin(kPi * j / n);
-        hl[slot] = s1 * s1 * 4 * v * v;
-      }
+      hl = hue_mm ? mm_lam(n, true, grid.axis_scale[0]) : per_lam(n, grid.axis_scale[0]);
       std::vector<T> hlT = toT(hl);
       o_cs = put(cs.data(), cs.size() * sizeof(T));
       o_hl = put(hlT.data(), n * sizeof(T));
       o_hld = put(hl.data(), n * sizeof(double));
-      hue_gemm = std::is_same<T, float>::value && n <= kHueGemmMax && B * P >= kHueGemmRows;
-      if (hue_gemm) {
-        // W[slot][i]: 1, cos / sin (2 pi i j / n) of frequency j = (slot + 1) / 2, (-1)^i (Nyquist slot of even n);
-        // the inverse, stored [i][slot], weighs the slots 1, 2, ..., 2, (1) and divides by n
-        std::vector<T> wf((size_t)n * n), wi((size_t)n * n);
-        for (int slot = 0; slot < n; ++slot) {
-          const bool nyq = n % 2 == 0 && slot == n - 1;
-          const int j = (slot + 1) / 2;
-          const double wgt = (slot == 0 || nyq) ? 1.0 : 2.0;
-          for (int i = 0; i < n; ++i) {
-            double v;
-            if (slot == 0) v = 1.0;
-            else if (nyq) v = (i & 1) ? -1.0 : 1.0;
-            else {
-              const double ang = 2 * kPi * (double)(((long long)i * j) % n) / n;
-              v = (slot & 1) ? std::cos(ang) : std::sin(ang);
-            }
-            wf[(size_t)slot * n + i] = (T)v;
-            wi[(size_t)i * n + slot] = (T)(wgt * v / n);
-          }
-        }
-        o_wf = put(wf.data(), wf.size() * sizeof(T));
-        o_wi = put(wi.data(), wi.size() * sizeof(T));
-        // the time DCT and its inverse as P x P matrices (rows of the padded tables above)
-        std::vector<T> mf((size_t)P * P), mi((size_t)P * P);
-        for (int r = 0; r < P; ++r)
-          for (int c = 0; c < P; ++c) {
-            mf[(size_t)r * P + c] = Mf[(size_t)r * pmax + c];
-            mi[(size_t)r * P + c] = Mi[(size_t)r * pmax + c];
-          }
-        o_mf = put(mf.data(), mf.size() * sizeof(T));
-        o_mi = put(mi.data(), mi.size() * sizeof(T));
-      }
     }
     CUDA_OK(cudaMalloc(&tabmem.p, h.size()));
     CUDA_OK(cudaMemcpy(tabmem.p, h.data(), h.size(), cudaMemcpyHostToDevice));
@@ -790,14 +822,6 @@ struct Plan final : PlanBase {
       for (const void* f : {(const void*)kmf, (const void*)kmi, (const void*)kmy})
         if (f) CUDA_OK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, maxsm));
     } else {
-      if (hue_gemm) {
-        CUDA_OK(cudaFuncSetAttribute((const void*)k_hue_tdiv, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)kHueTdivSmem));
-        hwf = (const T*)(base + o_wf);
-        hwi = (const T*)(base + o_wi);
-        hmf = (const T*)(base + o_mf);
-        hmi = (const T*)(base + o_mi);
-      }
       ht.cs = base + o_cs; ht.lam = base + o_hl; ht.lamd = (const double*)(base + o_hld);
       ht.lamt = base + o_lt; ht.lamtd = (const double*)(base + o_ltd);
       ht.Mt_f = base + o_Mf; ht.Mt_i = base + o_Mi;
@@ -813,6 +837,14 @@ struct Plan final : PlanBase {
       CUDA_OK(cudaFuncSetAttribute((const void*)k_hue_fwd<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxsm));
       CUDA_OK(cudaFuncSetAttribute((const void*)k_hue_inv<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxsm));
       CUDA_OK(cudaFuncSetAttribute((const void*)kh, cudaFuncAttributeMaxDynamicSharedMemorySize, maxsm));
+      if (hue_mm) {
+        mx.ft = (const T*)(base + o_mx[0]);
+        mx.it = (const T*)(base + o_mx[1]);
+        htt = (const T*)(base + o_tt);
+        for (const void* f : {(const void*)k_hue_x_fwd<T, true>, (const void*)k_hue_x_fwd<T, false>, (const void*)k_hue_x_inv<T, true>,
+                              (const void*)k_hue_x_inv<T, false>, (const void*)k_hue_tt<T, true>, (const void*)k_hue_tt<T, false>})
+          CUDA_OK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, maxsm));
+      }
     }
     return OT_OK;
   }
@@ -869,35 +901,22 @@ struct Plan final : PlanBase {
       if (evs) cudaEventRecord(evs[3], st);
     } else {
       if (evs) cudaEventRecord(evs[0], st);
-      const dim3 gg((n1 + 63) / 64, (B * P + 63) / 64);
-      if constexpr (std::is_same<T, float>::value) {
-        if (hue_gemm) {   // r into phi (overwritten by the inverse below), then R W^T into hat
-          k_hue_rhs<T><<<grid1d((long long)B * N), 256, 0, st>>>(g, asrc, f0n, f1n, phi);
-          k_gemm_nt<<<gg, 128, 0, st>>>(B * P, n1, n1, phi, hwf, hat);
-        }
+      if (hue_mm) {
+        launch_pdl(hue_small ? k_hue_x_fwd<T, true> : k_hue_x_fwd<T, false>, dim3((P + hf.rb - 1) / hf.rb, hf.nch, B),
+                   dim3(hf.nt), hf.smem, st, g, asrc, (const T*)f0n, (const T*)f1n, hat, mx, hf.rb, hf.chunk);
+        if (evs) cudaEventRecord(evs[1], st);
+        launch_pdl(hue_small ? k_hue_tt<T, true> : k_hue_tt<T, false>, dim3((n1 + hsc - 1) / hsc, B), dim3(256), smTt, st,
+                   g, hat, ht, htt);
+        if (evs) cudaEventRecord(evs[2], st);
+        launch_pdl(hue_small ? k_hue_x_inv<T, true> : k_hue_x_inv<T, false>, dim3((P + hi.rb - 1) / hi.rb, hi.nch, B),
+                   dim3(hi.nt), hi.smem, st, g, (const T*)hat, phi, mx, hi.rb, hi.chunk);
+      } else {
+        k_hue_fwd<T><<<dim3(P, B), 256, smH, st>>>(g, asrc, f0n, f1n, hat, ht);
+        if (evs) cudaEventRecord(evs[1], st);
+        kh<<<dim3((n1 + 256 / pmax - 1) / (256 / pmax), B), 256, smHt, st>>>(g, hat, ht);
+        if (evs) cudaEventRecord(evs[2], st);
+        k_hue_inv<T><<<dim3(P, B), 256, smH, st>>>(g, hat, phi, ht);
       }
-      if (!hue_gemm) k_hue_fwd<T><<<dim3(P, B), 256, smH, st>>>(g, asrc, f0n, f1n, hat, ht);
-      if (evs) cudaEventRecord(evs[1], st);
-      bool tdone = false;
-      if constexpr (std::is_same<T, float>::value) {
-        if (hue_gemm) {   // the time transforms of all slot columns: hat -> phi (with the divide) -> hat
-          const dim3 gt((n1 + 63) / 64, (P + 63) / 64, B);
-          if (P <= kHueTdivMaxP) {
-            k_hue_tdiv<<<dim3((n1 + 63) / 64, B), 256, kHueTdivSmem, st>>>(P, n1, (const float*)hmf,
-                                                                           (const float*)hmi, hat, (long long)P * n1, ht);
-          } else {
-            k_gemm_tn<true><<<gt, 256, 0, st>>>(P, n1, P, (const float*)hmf, hat, phi, (long long)P * n1, ht);
-            k_gemm_tn<false><<<gt, 256, 0, st>>>(P, n1, P, (const float*)hmi, phi, hat, (long long)P * n1, ht);
-          }
-          tdone = true;
-        }
-      }
-      if (!tdone) kh<<<dim3((n1 + 256 / pmax - 1) / (256 / pmax), B), 256, smHt, st>>>(g, hat, ht);
-      if (evs) cudaEventRecord(evs[2], st);
-      if constexpr (std::is_same<T, float>::value) {
-        if (hue_gemm) k_gemm_nt<<<gg, 128, 0, st>>>(B * P, n1, n1, hat, hwi, phi);
-      }
-      if (!hue_gemm) k_hue_inv<T><<<dim3(P, B), 256, smH, st>>>(g, hat, phi, ht);
       if (evs) cudaEventRecord(evs[3], st);
     }
   }
@@ -953,11 +972,9 @@ struct Plan final : PlanBase {
     }
     const dim3 grd((n1 + kThreadsUpd - 1) / kThreadsUpd, n2, C * P * B);
     if (check) {
-      if (wx) k_update<T, true, true><<<grd, kThreadsUpd, 0, st>>>(g, A, acc, mass);
-      else k_update<T, true, false><<<grd, kThreadsUpd, 0, st>>>(g, A, acc, mass);
+      launch_pdl(wx ? k_update<T, true, true> : k_update<T, true, false>, grd, dim3(kThreadsUpd), 0, st, g, A, acc, mass);
     } else {
-      if (wx) k_update<T, false, true><<<grd, kThreadsUpd, 0, st>>>(g, A, acc, mass);
-      else k_update<T, false, false><<<grd, kThreadsUpd, 0, st>>>(g, A, acc, mass);
+      launch_pdl(wx ? k_update<T, false, true> : k_update<T, false, false>, grd, dim3(kThreadsUpd), 0, st, g, A, acc, mass);
     }
   }
 

@@ -316,6 +316,7 @@ __global__ void __launch_bounds__(128) k_update(Geo<T> g, Arrays<T> A, double* _
   const int t = z % g.P;
   const int b = z / g.P;
   if (retired(g, b)) return;
+  pdl_wait();   // phi and the state are read from here on
   const bool live = x < g.n1;
   double r_db = 0, r_kx = 0, r_J = 0, r_m = 0, r_w = 0;
   if (live) {

@@ -45,22 +45,38 @@ def ot():
 @pytest.mark.parametrize("precision", [0, 2], ids=["f32", "f64"])
 @pytest.mark.parametrize("n,bc,P", GRIDS, ids=IDS)
 def test_projection(ot, n, bc, P, precision):
-    """Two problems in one plan: phi to 1e-5 (1e-6 in FP64, the float32 output) and x to the FP32 bound of A^T phi."""
-    plan = ot.Plan(ot.grid(n, bc, P, sigma=SIG, tau=TAU, precision=precision), batch=2)
+    _check_projection(ot, n, bc, P, precision, 2)
+
+
+HUES = [(2, 2, 1), (9, 3, 2), (101, 20, 3), (360, 64, 1), (722, 33, 2), (37, 13, 90), (250, 64, 40), (1001, 17, 70),
+        (3001, 8, 1)]
+
+
+@pytest.mark.parametrize("precision", [0, 2], ids=["f32", "f64"])
+@pytest.mark.parametrize("bins,P,batch", HUES)
+def test_hue_projection(ot, bins, P, batch, precision):
+    """Hue rows: sums in slices (few rows) and whole (many), chunks of slots, odd and even bins and P."""
+    _check_projection(ot, (bins,), (R,), P, precision, batch)
+
+
+def _check_projection(ot, n, bc, P, precision, batch):
+    """Problems 0 and batch - 1 of one plan: phi to 1e-5 (1e-6 in FP64, the float32 output) and x to the FP32 bound of
+    A^T phi."""
+    plan = ot.Plan(ot.grid(n, bc, P, sigma=SIG, tau=TAU, precision=precision), batch=batch)
     g = oracle_grid(n, bc, P)
     rng = np.random.default_rng(3)
     ins, refs, phis = [], [], []
-    for s in (4, 5):
+    for s in range(4, 4 + batch):
         f0, f1 = random_pair(g, s)
         am = [smooth_field(g.m_shape(k), rng).astype(np.float32).astype(np.float64) for k in range(g.d)]
         af = smooth_field(g.f_shape, rng).astype(np.float32).astype(np.float64)
-        m, f, phi = o.project(g, am, af, f0, f1)
         ins.append((f0, f1, pack_path(g, am, af)))
-        refs.append(pack_path(g, m, f))
+        m, f, phi = o.project(g, am, af, f0, f1) if s in (4, 3 + batch) else (None, None, None)
+        refs.append(pack_path(g, m, f) if m is not None else None)
         phis.append(phi)
     x, phi = plan.project(*(f32(np.stack([p[k] for p in ins])) for k in range(3)), with_phi=True)
-    x, phi = x.reshape(2, -1), phi.reshape(2, -1)
-    for i in range(2):
+    x, phi = x.reshape(batch, -1), phi.reshape(batch, -1)
+    for i in sorted({0, batch - 1}):
         tol = 1e-6 if precision == 2 else 1e-5
         assert rel(phi[i], phis[i].ravel()) <= tol
         assert rel(x[i], refs[i]) <= (tol if precision == 2 else correction_tolerance(g, phis[i], refs[i]))
