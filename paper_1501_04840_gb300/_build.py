@@ -14,7 +14,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libdynot.so")
-UNITS = (["api", "plan_f32", "plan_f64", "noalloc", "nn", "huepipe"] +
+UNITS = (["api", "plan_f32", "plan_f64", "noalloc", "nn", "huepipe", "sel_fft_f32", "sel_fftf_f32", "sel_ffti_f32"] +
          ["sel_%s_%s" % (k, t) for k in ("xt", "split", "yc", "mm", "upd") for t in ("f32", "f64")])
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ARCH + ["-O3", "-lineinfo", "-std=c++17", "--expt-relaxed-constexpr", "-Xcompiler", "-fPIC"]

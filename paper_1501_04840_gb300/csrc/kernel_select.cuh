@@ -9,7 +9,8 @@ namespace dynot {
 #ifdef SEL_XT
 template <typename T, int PM>
 KA<T> pick_ka_p(int n) {
-  switch (n) {
+  if constexpr (std::is_same<T, float>::value) return k_rhs_fwd_xt<T, 0, 0, PM>;   // FFT lengths: pick_kff
+  else switch (n) {
     case 64: return k_rhs_fwd_xt<T, 8, 8, PM>;
     case 96: return k_rhs_fwd_xt<T, 16, 6, PM>;
     case 128: return k_rhs_fwd_xt<T, 8, 16, PM>;
@@ -25,7 +26,8 @@ KA<T> pick_ka(int n, int pm) {
 }
 template <typename T, int PM>
 KC<T> pick_kc_p(int n) {
-  switch (n) {
+  if constexpr (std::is_same<T, float>::value) return k_inv_xt<T, 0, 0, PM>;       // FFT lengths: pick_kfi
+  else switch (n) {
     case 64: return k_inv_xt<T, 8, 8, PM>;
     case 96: return k_inv_xt<T, 16, 6, PM>;
     case 128: return k_inv_xt<T, 8, 16, PM>;
@@ -58,27 +60,75 @@ KCT<T> pick_kct(int pm) {
 #endif
 
 #ifdef SEL_YC
-template <typename T, int W>
-KB<T> pick_kb_w(int n) {
-  switch (n) {
-    case 64: return k_solve_yc<T, 8, 8, W, yc_nt(8, W)>;
-    case 96: return k_solve_yc<T, 16, 6, W, yc_nt(16, W)>;
-    case 128: return k_solve_yc<T, 8, 16, W, yc_nt(8, W)>;
-    case 192: return k_solve_yc<T, 16, 12, W, yc_nt(16, W)>;
-    case 256: return k_solve_yc<T, 16, 16, W, yc_nt(16, W)>;
-    case 512: return k_solve_yc<T, 16, 32, W, yc_nt(16, W)>;
+template <typename T>
+KB<T> pick_kb(int n) {
+  if constexpr (std::is_same<T, float>::value) return k_solve_yc<T, 0, 0, kW, 256>;   // FFT lengths: pick_kfy
+  else switch (n) {
+    case 64: return k_solve_yc<T, 8, 8, kW, yc_nt(8)>;
+    case 96: return k_solve_yc<T, 16, 6, kW, yc_nt(16)>;
+    case 128: return k_solve_yc<T, 8, 16, kW, yc_nt(8)>;
+    case 192: return k_solve_yc<T, 16, 12, kW, yc_nt(16)>;
+    case 256: return k_solve_yc<T, 16, 16, kW, yc_nt(16)>;
+    case 512: return k_solve_yc<T, 16, 32, kW, yc_nt(16)>;
     default: return k_solve_yc<T, 0, 0, kW, 256>;
   }
 }
-// strips of 4, 8 or 16 columns on the FFT lengths (FP32; the FP64 plan keeps 8)
-template <typename T>
-KB<T> pick_kb(int n, int w) {
-  if constexpr (std::is_same<T, float>::value) {
-    if (fft_len(n) && w == 4) return pick_kb_w<T, 4>(n);
-    if (fft_len(n) && w == 16) return pick_kb_w<T, 16>(n);
+#endif
+
+#ifdef SEL_FFT
+template <typename T, int C>
+KFY<T> pick_kfy_c(int n) {
+  switch (n) {
+    case 64: return k_fft_yc<T, 8, 8, C>;
+    case 96: return k_fft_yc<T, 16, 6, C>;
+    case 128: return k_fft_yc<T, 8, 16, C>;
+    case 192: return k_fft_yc<T, 16, 12, C>;
+    case 256: return k_fft_yc<T, 16, 16, C>;
+    case 512: return k_fft_yc<T, 16, 32, C>;
+    default: return nullptr;
   }
-  return pick_kb_w<T, kW>(n);
 }
+template <typename T>
+KFY<T> pick_kfy(int n, int C) {
+  switch (C) {
+    case 1: return pick_kfy_c<T, 1>(n);
+    case 2: return pick_kfy_c<T, 2>(n);
+    case 3: return pick_kfy_c<T, 3>(n);
+    default: return pick_kfy_c<T, 4>(n);
+  }
+}
+#endif
+
+#ifdef SEL_FFT_FWD
+template <int PM>
+KFF pick_kff_p(int n) {
+  switch (n) {
+    case 64: return k_fft_fwd_xt<8, 8, PM>;
+    case 96: return k_fft_fwd_xt<16, 6, PM>;
+    case 128: return k_fft_fwd_xt<8, 16, PM>;
+    case 192: return k_fft_fwd_xt<16, 12, PM>;
+    case 256: return k_fft_fwd_xt<16, 16, PM>;
+    case 512: return k_fft_fwd_xt<16, 32, PM>;
+    default: return nullptr;
+  }
+}
+KFF pick_kff(int n, int pm) { return pm == 16 ? pick_kff_p<16>(n) : (pm == 32 ? pick_kff_p<32>(n) : pick_kff_p<64>(n)); }
+#endif
+
+#ifdef SEL_FFT_INV
+template <int PM>
+KFI pick_kfi_p(int n) {
+  switch (n) {
+    case 64: return k_fft_inv_xt<8, 8, PM>;
+    case 96: return k_fft_inv_xt<16, 6, PM>;
+    case 128: return k_fft_inv_xt<8, 16, PM>;
+    case 192: return k_fft_inv_xt<16, 12, PM>;
+    case 256: return k_fft_inv_xt<16, 16, PM>;
+    case 512: return k_fft_inv_xt<16, 32, PM>;
+    default: return nullptr;
+  }
+}
+KFI pick_kfi(int n, int pm) { return pm == 16 ? pick_kfi_p<16>(n) : (pm == 32 ? pick_kfi_p<32>(n) : pick_kfi_p<64>(n)); }
 #endif
 
 #ifdef SEL_MM

@@ -107,7 +107,6 @@ struct Plan final : PlanBase {
   HueTables ht{};
   int pmax = 32;
   int scrA = 0, scrB = 0;
-  int yw = kW;              // column-strip width of the y/colour pass (autotuned on the FFT lengths)
   size_t smA = 0, smB = 0, smH = 0, smHt = 0;
   KA<T> ka = nullptr;
   KC<T> kc = nullptr;
@@ -117,6 +116,11 @@ struct Plan final : PlanBase {
   int scrS = 0;
   size_t smR = 0, smT = 0;
   KB<T> kb = nullptr;
+  size_t smY = 0, smF = 0;
+  KFF kff = nullptr;        // FP32, FFT lengths along x: the fused x/t passes
+  KFI kfi = nullptr;
+  FftXtTables ft{};
+  KFY<T> kfy = nullptr;     // FP32, FFT lengths along y: the fused y/colour pass
   KH<T> kh = nullptr;
   // transforms of axes without an FFT length as folded products
   bool x_mm = false, y_mm = false;
@@ -170,7 +174,7 @@ struct Plan final : PlanBase {
   size_t yc_smem() const {
     T *t0, *t1, *t2, *t3;
     c2<T> *c0, *c1, *c3;
-    return yc_layout<T>(nullptr, C, n2, yw, scrB, !y_fft(), &t0, &c0, &c1, &c3, &t1, &t2, &t3);
+    return yc_layout<T>(nullptr, C, n2, kW, scrB, !y_fft(), &t0, &c0, &c1, &c3, &t1, &t2, &t3);
   }
 
   ot_status init() override {
@@ -291,15 +295,13 @@ struct Plan final : PlanBase {
   }
 
   // Autotuner, run once per shape and device (the choice is cached for later plans of the shape):
-  //  - the y/colour pass: column strips of 4, 8 or 16 (FFT lengths, FP32) with 6, 12 or 24 row pairs per
-  //    FFT chunk;
   //  - the tiled update: staged by bulk tensor copies or with plain loads (where both exist), and time chunks
   //    of P, P/2, P/4 or P/8 planes, each timed over whole iterations (FP32).
   // Each candidate is timed over ten launches (after two untimed ones) on the zeroed workspace (b set so that the prox takes its
   // Newton branch); a later candidate must beat the best by 3 % (1 % for the FP32 update, timed over whole iterations,
   // where the update's share dilutes its differences; ties keep the earlier, simpler one).
   struct Tuned {
-    int yw = kW, tc = 0;
+    int tc = 0;
     bool tma = false;
   };
   static std::mutex& tune_mu() {
@@ -319,25 +321,6 @@ struct Plan final : PlanBase {
   bool tma_ok = false;      // tensor maps exist: the staged update is a candidate
   bool force_staged = false;
   bool plain_update = false;  // DYNOT_UPDATE_KERNEL=plain: no staged kernel, and hue batches update cell by cell
-
-  // y/colour pass with strips of w columns; false when its shared memory does not fit
-  bool set_yw(int w) {
-    if (hue) return false;
-    const int old = yw;
-    yw = w;
-    scrB = y_fft() ? (yc_threads(n2, yw) / fft_n1(n2)) * n2 : 4 * n2;
-    const size_t need = yc_smem();
-    int maxsm = 0;
-    if (cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) != cudaSuccess ||
-        (int)need > maxsm) {
-      yw = old;
-      scrB = y_fft() ? (yc_threads(n2, yw) / fft_n1(n2)) * n2 : 4 * n2;
-      return false;
-    }
-    smB = need;
-    kb = pick_kb<T>(y_fft() ? n2 : 0, yw);
-    return cudaFuncSetAttribute((const void*)kb, cudaFuncAttributeMaxDynamicSharedMemorySize, maxsm) == cudaSuccess;
-  }
 
   template <class F>
   ot_status time_launches(F&& launch, float& ms) {
@@ -366,7 +349,6 @@ struct Plan final : PlanBase {
       std::lock_guard<std::mutex> lk(tune_mu());
       auto it = tune_cache().find(key);
       if (it != tune_cache().end()) {
-        if (it->second.yw != yw) set_yw(it->second.yw);
         tc = it->second.tc;
         use_tma = it->second.tma;
         return OT_OK;
@@ -376,25 +358,9 @@ struct Plan final : PlanBase {
     const long long cells = (long long)B * N;
     k_fill<v4<T>><<<grid1d(cells), 256, 0, st>>>(cells, mk4<T>(T(0.5), T(0.5), T(0.5), T(1)), b[0]);
     CUDA_OK(cudaGetLastError());
-    if (!hue && y_fft() && std::is_same<T, float>::value) {
-      float best = 1e30f;
-      int bw = yw;
-      for (int w : {kW, 4, 16}) {
-        if (!set_yw(w)) continue;
-        float ms = 0;
-        OT_TRY(time_launches([&] {
-          launch_pdl(kb, dim3((n1 + yw - 1) / yw, P, B), dim3(yc_threads(n2, yw)), smB, st, g, hat, yc, scrB);
-        }, ms));
-        if (ms < 0.97f * best) {
-          best = ms;
-          bw = w;
-        }
-      }
-      set_yw(bw);
-    }
     if (tiled) {
       float best = 1e30f;
-      Tuned pick{yw, tc, use_tma};
+      Tuned pick{tc, use_tma};
       for (int kind = 0; kind < (tma_ok && !force_staged ? 2 : 1); ++kind) {
         use_tma = tma_ok && kind == 0;
         for (int c : cands) {
@@ -422,7 +388,7 @@ struct Plan final : PlanBase {
       CUDA_OK(cudaMemsetAsync(b[i], 0, (size_t)B * N * sizeof(v4<T>), st));
     }
     std::lock_guard<std::mutex> lk(tune_mu());
-    tune_cache()[key] = Tuned{yw, tc, use_tma};
+    tune_cache()[key] = Tuned{tc, use_tma};
     return OT_OK;
   }
   int tune_tc = 0;
@@ -679,9 +645,9 @@ struct Plan final : PlanBase {
       std::vector<T> c2v = g.per2 ? cs_pad(n2) : cos4(n2);
       o_c42 = put(c2v.data(), c2v.size() * sizeof(T));
       OT_TRY(choose_mm());
-      if (x_mm) {
-        mm_axis(mx, o_mx);
-        const int pm = mm_pm(P), ph = pm / 2, hP = (P + 1) / 2, P4 = (P + 3) / 4 * 4, hP4 = (hP + 3) / 4 * 4;
+      if (x_mm) mm_axis(mx, o_mx);
+      if (x_mm || (x_fft() && P < pmax)) {   // folded time transforms
+        const int pm = x_mm ? mm_pm(P) : pmax, ph = pm / 2, hP = (P + 1) / 2, P4 = (P + 3) / 4 * 4, hP4 = (hP + 3) / 4 * 4;
         std::vector<T> tf((size_t)P4 * ph, T(0)), ti((size_t)hP4 * pm, T(0));
         for (int k = 0; k < P; ++k)
           for (int t = 0; t < P; ++t) {
@@ -776,17 +742,17 @@ struct Plan final : PlanBase {
         ax.ft = (const T*)(base + off[0]);
         ax.it = (const T*)(base + off[1]);
       };
-      if (x_mm) {
-        mm_ptrs(mx, o_mx);
-        mtf = (const T*)(base + o_mtf);
-        mti = (const T*)(base + o_mti);
-      }
+      if (x_mm) mm_ptrs(mx, o_mx);
+      mtf = (const T*)(base + o_mtf);
+      mti = (const T*)(base + o_mti);
       if (y_mm) mm_ptrs(my, o_my);
       scrA = x_fft() ? (kThreadsXt / fft_n1(n1)) * n1 : 4 * n1;
-      scrB = y_fft() ? (yc_threads(n2, yw) / fft_n1(n2)) * n2 : 4 * n2;
+      scrB = y_fft() ? (yc_threads(n2) / fft_n1(n2)) * n2 : 4 * n2;
       ka = pick_ka<T>(x_fft() ? n1 : 0, pmax);
       kc = pick_kc<T>(x_fft() ? n1 : 0, pmax);
       kb = pick_kb<T>(y_fft() ? n2 : 0);
+      if constexpr (std::is_same<T, float>::value) kfy = y_fft() ? pick_kfy<T>(n2, C) : nullptr;
+      if (kfy) smY = fft_yc_smem<T>(fft_n1(n2), n2 / fft_n1(n2), C);
       smA = xt_smem();
       smB = yc_smem();
       int maxsm = 0;
@@ -805,6 +771,16 @@ struct Plan final : PlanBase {
         krx_i = pick_krx<T, true>(x_fft() ? n1 : 0);
         kct = pick_kct<T>(pmax);
       }
+      if constexpr (std::is_same<T, float>::value) {
+        if (x_fft() && !split_xt) {
+          kff = pick_kff(n1, pmax);
+          kfi = pick_kfi(n1, pmax);
+          smF = fft_xt_smem(n1, P, pmax);
+          ft = FftXtTables{(const float2*)xt.tw, (const float2*)xt.hw, (const float2*)xt.twt, (const float2*)xt.hwt, mtf, mti};
+          CUDA_OK(cudaFuncSetAttribute((const void*)kff, cudaFuncAttributeMaxDynamicSharedMemorySize, maxsm));
+          CUDA_OK(cudaFuncSetAttribute((const void*)kfi, cudaFuncAttributeMaxDynamicSharedMemorySize, maxsm));
+        }
+      }
       if ((!split_xt && (int)smA > maxsm) || (int)smB > maxsm || (split_xt && ((int)smR > maxsm || (int)smT > maxsm)))
         return seterr(OT_EUNSUPPORTED, "grid needs %zu / %zu bytes of shared memory per block (max %d)",
                       split_xt ? std::max(smR, smT) : smA, smB, maxsm);
@@ -819,7 +795,7 @@ struct Plan final : PlanBase {
         CUDA_OK(cudaFuncSetAttribute((const void*)kc, cudaFuncAttributeMaxDynamicSharedMemorySize, maxsm));
       }
       CUDA_OK(cudaFuncSetAttribute((const void*)kb, cudaFuncAttributeMaxDynamicSharedMemorySize, maxsm));
-      for (const void* f : {(const void*)kmf, (const void*)kmi, (const void*)kmy})
+      for (const void* f : {(const void*)kmf, (const void*)kmi, (const void*)kmy, (const void*)kfy})
         if (f) CUDA_OK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, maxsm));
     } else {
       ht.cs = base + o_cs; ht.lam = base + o_hl; ht.lamd = (const double*)(base + o_hld);
@@ -869,7 +845,16 @@ struct Plan final : PlanBase {
   void enqueue_poisson_src(const v4<T>* asrc, cudaEvent_t* evs) {
     if (!hue) {
       if (evs) cudaEventRecord(evs[0], st);
-      if (x_mm) {
+      bool done = false;
+      if constexpr (std::is_same<T, float>::value) {
+        if (kff) {
+          launch_pdl(kff, dim3(n2, C, B), dim3(fft_xt_threads(n1, pmax)), smF, st, g, asrc, (const T*)f0n, (const T*)f1n,
+                     hat, ft);
+          done = true;
+        }
+      }
+      if (done) {
+      } else if (x_mm) {
         launch_pdl(kmf, dim3(n2, C, B), dim3(ntMf), smMx, st, g, asrc, (const T*)f0n, (const T*)f1n, hat, mx, mtf);
       } else if (split_xt) {
         k_rhs_cells<T><<<grid1d((long long)B * N), 256, 0, st>>>(g, asrc, (const T*)f0n, (const T*)f1n, hat);
@@ -882,13 +867,18 @@ struct Plan final : PlanBase {
                    scrA);
       }
       if (evs) cudaEventRecord(evs[1], st);
-      if (y_mm)
+      if (kfy)
+        launch_pdl(kfy, dim3((n1 + fft_yc_w(C) - 1) / fft_yc_w(C), P, B), dim3(kFftNP * fft_n1(n2)), smY, st, g, hat, yc);
+      else if (y_mm)
         launch_pdl(kmy, dim3((n1 + wMy - 1) / wMy, P, B), dim3(ntMy), smMy, st, g, hat, yc, my, wMy);
       else
-        launch_pdl(kb, dim3((n1 + yw - 1) / yw, P, B), dim3(yc_threads(y_fft() ? n2 : 0, yw)), smB, st, g, hat, yc,
+        launch_pdl(kb, dim3((n1 + kW - 1) / kW, P, B), dim3(yc_threads(y_fft() ? n2 : 0)), smB, st, g, hat, yc,
                    scrB);
       if (evs) cudaEventRecord(evs[2], st);
-      if (x_mm) {
+      if constexpr (std::is_same<T, float>::value)
+        if (kfi) launch_pdl(kfi, dim3(n2, C, B), dim3(fft_xt_threads(n1, pmax)), smF, st, g, (const T*)hat, phi, ft);
+      if (done) {
+      } else if (x_mm) {
         launch_pdl(kmi, dim3(n2, C, B), dim3(ntMi), smMi, st, g, (const T*)hat, phi, mx, mti);
       } else if (split_xt) {
         launch_pdl(kct, dim3((n1 + kColsT - 1) / kColsT, n2 * C, B), dim3(kColsT), smT, st, g, hat,

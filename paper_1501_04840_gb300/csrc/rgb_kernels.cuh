@@ -479,7 +479,8 @@ __device__ __forceinline__ void store_tile_rows(const T* tile, T* __restrict__ d
     for (int x = threadIdx.x; x < n1; x += blockDim.x) dst[(size_t)t * S + x] = tile[t * n1 + x];
 }
 
-// N1 == 0 selects the dense x transform.
+// N1 == 0 selects the dense x transform.  FP32 plans take k_fft_fwd_xt (fft_kernels.cuh) on FFT lengths and
+// k_mm_fwd_xt (mm_kernels.cuh) on others; this kernel serves the FP64 plan and FP32 planes that fit neither.
 template <typename T, int N1, int N2, int PMAX>
 __global__ void __launch_bounds__(256, DYNOT_XT_MINB) k_rhs_fwd_xt(Geo<T> g, const v4<T>* __restrict__ ap,
                                                     const T* __restrict__ f0, const T* __restrict__ f1,

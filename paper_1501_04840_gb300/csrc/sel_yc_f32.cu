@@ -2,5 +2,5 @@
 #include "kernel_select.cuh"
 
 namespace dynot {
-template KB<float> pick_kb<float>(int, int);
+template KB<float> pick_kb<float>(int);
 }  // namespace dynot

@@ -2,5 +2,5 @@
 #include "kernel_select.cuh"
 
 namespace dynot {
-template KB<double> pick_kb<double>(int, int);
+template KB<double> pick_kb<double>(int);
 }  // namespace dynot

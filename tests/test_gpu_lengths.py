@@ -1,5 +1,5 @@
-"""GPU parity of the transforms for axis lengths without an FFT (folded products, csrc/mm_kernels.cuh) against the
-FP64 oracle: one projection and one iteration per grid, with the tolerances of test_gpu_parity.  The grids sit at the
+"""GPU parity of the transforms over axis lengths (folded products, csrc/mm_kernels.cuh; fused FFT passes,
+csrc/fft_kernels.cuh) against the FP64 oracle: one projection and one iteration per grid, with the tolerances of test_gpu_parity.  The grids sit at the
 kernels' edges: lengths around whole groups of four outputs and eight time planes, one to four channels, odd and short
 axes, P beside each register width, periodic axes with and without a Nyquist slot, and both precisions."""
 import numpy as np
@@ -26,6 +26,15 @@ GRIDS = [
     ((128, 100, 1), (N, N, N), 16),
     ((130, 7, 3), RGB, 49),
     ((2, 515, 3), RGB, 6),
+    # FFT lengths (csrc/fft_kernels.cuh): every length on either axis, channels, and time lengths that fill, leave or
+    # exceed a register transform
+    ((512, 64, 3), RGB, 64),
+    ((64, 512, 2), (N, N, N), 20),
+    ((96, 96, 4), (R, N, R), 40),
+    ((192, 128, 1), (N, R, N), 63),
+    ((256, 192), (R, R), 16),
+    ((512, 30), (R, N), 15),
+    ((33, 256, 3), RGB, 3),
 ]
 IDS = ["x".join(map(str, n)) + "_" + "".join(b[0] for b in bc) + "_P%d" % P for n, bc, P in GRIDS]
 
