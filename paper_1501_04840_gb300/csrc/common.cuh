@@ -156,4 +156,33 @@ struct KSum {
   }
 };
 
+// A sum carried in two values of the working precision: every addition keeps its rounding error (Knuth's two-sum) and
+// every product its own (a fused multiply-add), so FP32 terms and sums are good to about 2^-45.  The FP64 pipe is a
+// sixty-fourth of the FP32 one: five FP64 additions per warp and plane took longer than the rest of a residual check.
+template <typename T>
+struct Sum2 {
+  T hi = T(0), lo = T(0);
+  __device__ __forceinline__ void add(T v) {
+    const T s = hi + v, b = s - hi;
+    lo += (hi - (s - b)) + (v - b);
+    hi = s;
+  }
+  __device__ __forceinline__ void add_product(T a, T b) {
+    const T p = a * b;
+    lo += fma(a, b, -p);
+    add(p);
+  }
+  // the sum over the lanes of a warp, in every lane
+  __device__ __forceinline__ double warp_total() const {
+    Sum2 t = *this;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const T h = __shfl_xor_sync(0xffffffffu, t.hi, o), l = __shfl_xor_sync(0xffffffffu, t.lo, o);
+      t.add(h);
+      t.lo += l;
+    }
+    return (double)t.hi + (double)t.lo;
+  }
+};
+
 }  // namespace dynot

@@ -97,9 +97,16 @@ struct Plan final : PlanBase {
   int* err = nullptr;       // set by a kernel whose bounded device wait ran out (sticky until the next start)
   int* active = nullptr;    // [B] per-problem flags of a retiring batch (g.active points here once enabled)
   std::vector<int> h_active;
-  int* h_err = nullptr;     // pinned host copy, read with the residuals
-  double* h_acc = nullptr;  // pinned host copies of acc and mass
+  // pinned host copies of acc, mass and err, which lie side by side on either side: one copy per check
+  double* h_acc = nullptr;
   double* h_mass = nullptr;
+  int* h_err = nullptr;
+  size_t res_bytes() const { return sizeof(double) * B * kAcc + rnd16(sizeof(double) * (size_t)B * P) + sizeof(int); }
+  cudaError_t copy_results() { return cudaMemcpyAsync(h_acc, acc, res_bytes(), cudaMemcpyDeviceToHost, st); }
+  // the sums that the per-cell update adds to (the tiled ones write theirs whole)
+  cudaError_t clear_results() {
+    return tiled ? cudaSuccess : cudaMemsetAsync(acc, 0, sizeof(double) * B * (kAcc + (size_t)P), st);
+  }
   // transform tables
   DevMem tabmem;
   XtTables xt{};
@@ -162,8 +169,6 @@ struct Plan final : PlanBase {
     for (auto& e : ev)
       if (e) cudaEventDestroy(e);
     if (h_acc) cudaFreeHost(h_acc);
-    if (h_err) cudaFreeHost(h_err);
-    if (h_mass) cudaFreeHost(h_mass);
   }
 
   // the FFT paths cover power-of-two axes (DCT for Neumann, real Fourier slots for periodic ones);
@@ -215,19 +220,19 @@ struct Plan final : PlanBase {
     stage = (float*)take(stage_floats * sizeof(float));
     acc = (double*)take(sizeof(double) * B * kAcc);
     mass = (double*)take(sizeof(double) * (size_t)B * P);
+    err = (int*)take(sizeof(int));
     chk = (double*)take(sizeof(double) * B * kChk);
     scl = (double*)take(sizeof(double) * B * 2);
     part = (double*)take(part_bytes());
-    err = (int*)take(sizeof(int));
     active = (int*)take(sizeof(int) * B);
     CUDA_OK(cudaMemsetAsync(mem.p, 0, bytes, st));
 
     OT_TRY(build_tables());
     for (auto& e : ev) CUDA_OK(cudaEventCreate(&e));
-    CUDA_OK(cudaMallocHost(&h_acc, sizeof(double) * B * kAcc));
-    CUDA_OK(cudaMallocHost(&h_err, sizeof(int)));
+    CUDA_OK(cudaMallocHost(&h_acc, res_bytes()));
+    h_mass = h_acc + (size_t)B * kAcc;
+    h_err = (int*)((char*)h_mass + rnd16(sizeof(double) * (size_t)B * P));
     *h_err = 0;
-    CUDA_OK(cudaMallocHost(&h_mass, sizeof(double) * (size_t)B * P));
     out_scale.assign(B, 1.0);
     tiled = !hue && C <= 4;
     {
@@ -941,7 +946,9 @@ struct Plan final : PlanBase {
         const TileLayout Lt{S, n1, n1 * n2, (long long)P * S, n1, (long long)S};
         launch_pdl(pick_kd<T>(C, check, wx, g.per1 || g.per2), grd, dim3(kTX, kTY), 0, st, g, A, tc, Lt, part);
       }
-      if (check) k_reduce_check<<<B, 512, 0, st>>>(part, (int)(grd.x * grd.y * grd.z / B), P, acc, mass, g.active);
+      if (check)
+        k_reduce_check<<<dim3((4 + P + kReduceThreads / 32 - 1) / (kReduceThreads / 32), B), kReduceThreads, 0, st>>>(
+            part, (int)(grd.x * grd.y * grd.z / B), P, acc, mass, g.active);
       return;
     }
     if (hue && !check && !wx && !g.active && B >= 8 && !plain_update) {
@@ -1014,15 +1021,12 @@ struct Plan final : PlanBase {
 
   // one iteration with residuals (and x output); results land in pinned host memory
   ot_status enqueue_check(bool wx) {
-    CUDA_OK(cudaMemsetAsync(acc, 0, sizeof(double) * B * kAcc, st));
-    CUDA_OK(cudaMemsetAsync(mass, 0, sizeof(double) * (size_t)B * P, st));
+    CUDA_OK(clear_results());
     enqueue_iteration(par, true, wx);
     CUDA_OK(cudaGetLastError());
     par ^= 1;
     if (wx) have_x = true;
-    CUDA_OK(cudaMemcpyAsync(h_acc, acc, sizeof(double) * B * kAcc, cudaMemcpyDeviceToHost, st));
-    CUDA_OK(cudaMemcpyAsync(h_mass, mass, sizeof(double) * (size_t)B * P, cudaMemcpyDeviceToHost, st));
-    CUDA_OK(cudaMemcpyAsync(h_err, err, sizeof(int), cudaMemcpyDeviceToHost, st));
+    CUDA_OK(copy_results());
     return OT_OK;
   }
 
@@ -1059,13 +1063,10 @@ struct Plan final : PlanBase {
     if (gcheck[p][lead]) return OT_OK;
     cudaGraph_t gr = nullptr;
     CUDA_OK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-    cudaMemsetAsync(acc, 0, sizeof(double) * B * kAcc, st);
-    cudaMemsetAsync(mass, 0, sizeof(double) * (size_t)B * P, st);
+    clear_results();
     if (lead) enqueue_iteration(p, false, false);
     enqueue_iteration(lead ? 1 - p : p, true, true);
-    cudaMemcpyAsync(h_acc, acc, sizeof(double) * B * kAcc, cudaMemcpyDeviceToHost, st);
-    cudaMemcpyAsync(h_mass, mass, sizeof(double) * (size_t)B * P, cudaMemcpyDeviceToHost, st);
-    cudaMemcpyAsync(h_err, err, sizeof(int), cudaMemcpyDeviceToHost, st);
+    copy_results();
     const cudaError_t le = cudaGetLastError();
     cudaError_t e = cudaStreamEndCapture(st, &gr);
     if (le != cudaSuccess) {

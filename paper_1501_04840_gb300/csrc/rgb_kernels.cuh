@@ -298,13 +298,6 @@ struct CellCtx {
 //   mass[b*P + t]: sum over space of f at time (t+1)/P
 constexpr int kAcc = 4;
 
-template <typename T>
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
 template <typename T, bool CHECK, bool WRITE_X>
 __global__ void __launch_bounds__(128) k_update(Geo<T> g, Arrays<T> A, double* __restrict__ acc,
                                                 double* __restrict__ mass) {
@@ -318,7 +311,7 @@ __global__ void __launch_bounds__(128) k_update(Geo<T> g, Arrays<T> A, double* _
   if (retired(g, b)) return;
   pdl_wait();   // phi and the state are read from here on
   const bool live = x < g.n1;
-  double r_db = 0, r_kx = 0, r_J = 0, r_m = 0, r_w = 0;
+  Sum2<T> r_db, r_kx, r_J, r_m, r_w;
   if (live) {
     CellCtx<T> cc{g, A, b};
     T bb[4], bn[4], xrr[4], kx[4], U0, U1, U2, V;
@@ -356,34 +349,35 @@ __global__ void __launch_bounds__(128) k_update(Geo<T> g, Arrays<T> A, double* _
     if (CHECK) {
       const v4<T> bo4 = A.b[i0];
       const T bo[4] = {bo4.x, bo4.y, bo4.z, bo4.w};
+      const v4<T> wv = A.w[i0];
+      const T wk[4] = {wv.x, wv.y, wv.z, wv.w};
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        const double db = (double)bn[k] - (double)bo[k];
-        r_db += db * db;
-        r_kx += (double)kx[k] * (double)kx[k];
+        const T db = bn[k] - bo[k];
+        r_db.add_product(db, db);
+        r_kx.add_product(kx[k], kx[k]);
+        r_w.add_product(bn[k], wk[k]);
       }
-      const double uu = (double)U0 * U0 + (double)U1 * U1 + (double)U2 * U2;
-      if (V > T(0)) r_J = uu / (2.0 * (double)V);
-      r_m = (double)xrr[3];
-      const v4<T> wv = A.w[i0];
-      r_w = (double)bn[0] * wv.x + (double)bn[1] * wv.y + (double)bn[2] * wv.z + (double)bn[3] * wv.w;
+      if (V > T(0)) {
+        // |u|^2 / (2 v), the quotient with its remainder
+        Sum2<T> uu;
+        uu.add_product(U0, U0);
+        uu.add_product(U1, U1);
+        uu.add_product(U2, U2);
+        const T v2 = T(2) * V, q = uu.hi / v2;
+        r_J.hi = q;
+        r_J.lo = (fma(-q, v2, uu.hi) + uu.lo) / v2;
+      }
+      r_m.add(xrr[3]);
     }
   }
   if (CHECK) {
     __shared__ double red[4][5];
-    r_db = warp_sum<T>(r_db);
-    r_kx = warp_sum<T>(r_kx);
-    r_J = warp_sum<T>(r_J);
-    r_m = warp_sum<T>(r_m);
-    r_w = warp_sum<T>(r_w);
+    const double d[5] = {r_db.warp_total(), r_kx.warp_total(), r_J.warp_total(), r_m.warp_total(), r_w.warp_total()};
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    if (l == 0) {
-      red[w][0] = r_db;
-      red[w][1] = r_kx;
-      red[w][2] = r_J;
-      red[w][3] = r_m;
-      red[w][4] = r_w;
-    }
+    if (l == 0)
+#pragma unroll
+      for (int q = 0; q < 5; ++q) red[w][q] = d[q];
     __syncthreads();
     if (threadIdx.x < 5) {
       double s = 0;
@@ -917,7 +911,7 @@ constexpr int kTX = 32, kTY = 8;
 #define DYNOT_UPD_MINB 3   // blocks per SM the tiled update is compiled for
 #endif
 
-// Per-block partial sums of the residual check: [problem][block][kPart] with
+// Per-block partial sums of the residual check: [problem][kPart][block] with
 // 0: |b+ - b|^2, 1: |K x + (0, f_b^+)|^2, 2: J(u, v), 3 + t: mass of the time slice t (t < 64),
 // kPartW = 67: <b+, w> (the dual value over sigma).
 constexpr int kPart = 68;
@@ -935,19 +929,21 @@ struct TileLayout {
 };
 
 // Per-block partial sums of a check (called by every thread of a 32 x 8 block after its plane loop):
-// FP64 sums of the threads' compensated partials, written to part[problem][block][...].
+// sums of the threads' compensated partials (two-value sums in a warp, FP64 across warps), written to
+// part[problem][quantity][block].
 template <typename T>
 __device__ __forceinline__ void block_check_partials(const KSum<T>& r_db, const KSum<T>& r_kx, const KSum<T>& r_J,
                                                      const KSum<T>& r_w, int lane, int row, int nch, int b, int t0,
                                                      int tend, int P, double* __restrict__ part,
                                                      const double (&smass)[64]) {
   __shared__ double red[kTY][4];
-  double d[4] = {(double)r_db.s - (double)r_db.c, (double)r_kx.s - (double)r_kx.c, (double)r_J.s - (double)r_J.c,
-                 (double)r_w.s - (double)r_w.c};
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) d[q] += __shfl_xor_sync(0xffffffffu, d[q], o);
+  auto total = [](const KSum<T>& k) {
+    Sum2<T> t;
+    t.hi = k.s;
+    t.lo = -k.c;
+    return t.warp_total();
+  };
+  const double d[4] = {total(r_db), total(r_kx), total(r_J), total(r_w)};
   if (lane == 0)
 #pragma unroll
     for (int q = 0; q < 4; ++q) red[row][q] = d[q];
@@ -955,13 +951,13 @@ __device__ __forceinline__ void block_check_partials(const KSum<T>& r_db, const 
   const int tid = lane + kTX * row;
   const int nblk = gridDim.x * gridDim.y * nch;    // blocks of one problem
   const int jb = ((blockIdx.z % nch) * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-  double* pp = part + ((size_t)b * nblk + jb) * kPart;
+  double* pp = part + (size_t)b * nblk * kPart + jb;   // quantity q at pp[q * nblk]
   if (tid < 4) {
     double sum = 0;
     for (int i = 0; i < kTY; ++i) sum += red[i][tid];
-    pp[tid < 3 ? tid : kPartW] = sum;
+    pp[(size_t)(tid < 3 ? tid : kPartW) * nblk] = sum;
   }
-  for (int t = tid; t < 64; t += kTX * kTY) pp[3 + t] = (t >= t0 && t < tend && t < P - 1) ? smass[t] : 0.0;
+  for (int t = tid; t < P; t += kTX * kTY) pp[(size_t)(3 + t) * nblk] = (t >= t0 && t < tend && t < P - 1) ? smass[t] : 0.0;
 }
 
 // The body of the tiled update.  INTERIOR: every thread of the block has both x and y neighbours
@@ -1148,9 +1144,9 @@ __device__ __forceinline__ void update_tiled_body(const Geo<T>& g, const Arrays<
 #pragma unroll
           for (int c = 0; c < C; ++c) mt += xr[c][3];
         }
-        double m = (double)mt;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
+        Sum2<T> ms;
+        ms.hi = mt;
+        const double m = ms.warp_total();
         if (lane == 0) atomicAdd(&smass[t], m);
       }
     }
@@ -1185,25 +1181,27 @@ __global__ void __launch_bounds__(kTX * kTY, DYNOT_UPD_MINB) k_update_tiled(Geo<
 }
 
 
-// Sum the per-block partials of each problem (one block per problem) into acc and mass: one warp per quantity
-// (the 3 residual and energy terms, the P mass sums, the dual term), lanes striding over the blocks in a fixed order.
-static __global__ void k_reduce_check(const double* __restrict__ part, int nblk, int P, double* __restrict__ acc,
-                               double* __restrict__ mass, const int* __restrict__ active) {
-  const int b = blockIdx.x;
-  if (active != nullptr && active[b] == 0) return;
-  const double* pb = part + (size_t)b * nblk * kPart;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  for (int qi = warp; qi < 4 + P; qi += nw) {
-    const int q = qi < 3 + P ? qi : kPartW;
-    double s = 0;
-    for (int j = lane; j < nblk; j += 32) s += pb[(size_t)j * kPart + q];
+// Sum the per-block partials of each problem (blocks of 8 warps, problem blockIdx.y) into acc and mass: one warp per
+// quantity (the 3 residual and energy terms, the P mass sums, the dual term), lanes striding over the blocks in a fixed
+// order.  2664 partials of 36 quantities: 33 us as one block reading [block][quantity], 5 us like this.
+constexpr int kReduceThreads = 256;
+static __global__ void __launch_bounds__(kReduceThreads) k_reduce_check(const double* __restrict__ part, int nblk, int P,
+                                                                        double* __restrict__ acc, double* __restrict__ mass,
+                                                                        const int* __restrict__ active) {
+  const int b = blockIdx.y, lane = threadIdx.x & 31;
+  const int qi = blockIdx.x * (kReduceThreads / 32) + (threadIdx.x >> 5);
+  if (qi >= 4 + P || (active != nullptr && active[b] == 0)) return;
+  const int q = qi < 3 + P ? qi : kPartW;
+  const double* pq = part + (size_t)b * nblk * kPart + (size_t)q * nblk;
+  double s = 0;
+#pragma unroll 8
+  for (int j = lane; j < nblk; j += 32) s += pq[j];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) {
-      if (q < 3) acc[(size_t)b * kAcc + q] = s;
-      else if (q == kPartW) acc[(size_t)b * kAcc + 3] = s;
-      else if (q - 3 < P) mass[(size_t)b * P + (q - 3)] = s;
-    }
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) {
+    if (q < 3) acc[(size_t)b * kAcc + q] = s;
+    else if (q == kPartW) acc[(size_t)b * kAcc + 3] = s;
+    else mass[(size_t)b * P + (q - 3)] = s;
   }
 }
 

@@ -299,9 +299,9 @@ __device__ __forceinline__ void update_tma_body(const Geo<float>& g, const Array
 #pragma unroll
           for (int c = 0; c < C; ++c) mt += xr[c][3];
         }
-        double m = (double)mt;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
+        Sum2<float> ms;
+        ms.hi = mt;
+        const double m = ms.warp_total();
         if (lane == 0) atomicAdd(&smass[t], m);
       }
     }
