@@ -12,8 +12,8 @@
 // the same steps backwards: M2-point DFTs over k2, twiddles, M1-point DFTs over k1.
 //
 // Against the row-based passes of rgb_kernels.cuh (which unpacked every spectrum to rows and back), per launch from
-// events on one GB300: 256x256x3, P = 32: y/colour 46.8 -> 28.1 us, inverse x/t 32.8 -> 20.5, forward x/t 58.8 -> 47.6;
-// 512x512x3, P = 64 (whose time transform was a dense product): 432 -> 217, 587 -> 147, 886 -> 368 us; 128x128x3, P = 32:
+// events on one GB300: 256x256x3, P = 32: y/colour 46.8 -> 28.1 us, inverse x/t 32.8 -> 20.5, forward x/t 58.8 -> 41.4;
+// 512x512x3, P = 64 (whose time transform was a dense product): 432 -> 217, 587 -> 147, 886 -> 284 us; 128x128x3, P = 32:
 // 21.4 -> 16.1, 14.3 -> 10.1, 21.7 -> 15.1 us.  Shared-memory accesses fall to about a third; the y/colour pass is left
 // with issue and the barriers of its five passes, the forward x/t pass with the L2 traffic of forming r (a 16-byte
 // cell and two neighbours' cells for 4 bytes of each).
@@ -416,12 +416,14 @@ __device__ __forceinline__ void idct_reg(float (&x)[P], const float2* tw, const 
 
 template <int M1, int M2, int PM>
 __global__ void __launch_bounds__((fft_xt_nt<M1 * M2, PM>()), (fft_xt_minb<M1 * M2, PM>()))
-    k_fft_fwd_xt(Geo<float> g, const float4* __restrict__ ap, const float* __restrict__ f0,
+    k_fft_fwd_xt(Geo<float> g, const float4* __restrict__ ap, const float* __restrict__ f0,   // grid (C, n2, B)
                  const float* __restrict__ f1, float* __restrict__ hat, FftXtTables tb) {
   using L = FftXt<PM>;
   constexpr int N = M1 * M2, NT = fft_xt_nt<N, PM>(), PC = L::PC, ST = L::ST, NCH = L::NCH, PH = PM / 2;
   extern __shared__ __align__(16) char smraw[];
-  const int y = blockIdx.x, c = blockIdx.y, b = blockIdx.z, tid = threadIdx.x;
+  // channels run fastest: the row of channel c - 1, whose faces this block reads, is then in L2 (with y fastest it had
+  // left it at large grids: 368 against 284 us at 512x512x3, P = 64; 47.6 against 41.4 at 256x256x3, P = 32)
+  const int c = blockIdx.x, y = blockIdx.y, b = blockIdx.z, tid = threadIdx.x;
   if (retired(g, b)) return;
   const int P = g.P;
   const bool per = g.per1, tfft = P == PM;

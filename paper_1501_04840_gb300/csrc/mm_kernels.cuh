@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(kMmXtThreads, sizeof(T) == 4 ? 2 : 1)
                 T* __restrict__ hat, MmAxis<T> ax, const T* __restrict__ Mtg) {
   constexpr int PH = PM / 2;
   extern __shared__ __align__(16) char smraw[];
-  const int y = blockIdx.x, c = blockIdx.y, b = blockIdx.z;
+  const int c = blockIdx.x, y = blockIdx.y, b = blockIdx.z;
   if (retired(g, b)) return;
   const int n1 = g.n1, P = g.P, ld = mm_ldt(P), P4 = (P + 3) / 4 * 4, hP = (P + 1) / 2;
   T* X = (T*)smraw;          // [x][t]

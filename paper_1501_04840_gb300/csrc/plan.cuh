@@ -477,9 +477,9 @@ struct Plan final : PlanBase {
       for (int w = 16; w >= wt; w /= 2) {
         const int items = mm_yc_items(my.lf, C, w);
         const size_t sm = mm_yc_smem<T>(n2, C, w, bufy);
-        // narrower strips while the grid has fewer than four blocks per SM (180x135x3x24: 40.0 us with 8 columns, 42.5
+        // narrower strips while the grid has fewer than three blocks per SM (180x135x3x24: 40.0 us with 8 columns, 42.5
         // with 16; 300x200x3x16: 63.2 against 67.2)
-        const bool more = w > wt && (long long)((n1 + w - 1) / w) * P * B < 4 * 152;
+        const bool more = w > wt && (long long)((n1 + w - 1) / w) * P * B < 3 * 152;
         if (items > kMmYcThreads || (int)sm > maxsm || more) continue;
         y_mm = true;
         wMy = w;
@@ -853,14 +853,14 @@ struct Plan final : PlanBase {
       bool done = false;
       if constexpr (std::is_same<T, float>::value) {
         if (kff) {
-          launch_pdl(kff, dim3(n2, C, B), dim3(fft_xt_threads(n1, pmax)), smF, st, g, asrc, (const T*)f0n, (const T*)f1n,
+          launch_pdl(kff, dim3(C, n2, B), dim3(fft_xt_threads(n1, pmax)), smF, st, g, asrc, (const T*)f0n, (const T*)f1n,
                      hat, ft);
           done = true;
         }
       }
       if (done) {
       } else if (x_mm) {
-        launch_pdl(kmf, dim3(n2, C, B), dim3(ntMf), smMx, st, g, asrc, (const T*)f0n, (const T*)f1n, hat, mx, mtf);
+        launch_pdl(kmf, dim3(C, n2, B), dim3(ntMf), smMx, st, g, asrc, (const T*)f0n, (const T*)f1n, hat, mx, mtf);
       } else if (split_xt) {
         k_rhs_cells<T><<<grid1d((long long)B * N), 256, 0, st>>>(g, asrc, (const T*)f0n, (const T*)f1n, hat);
         launch_pdl(krx_f, dim3((P + kRowsX - 1) / kRowsX, n2 * C, B), dim3(256), smR, st, g, (const T*)hat, hat, xt,
