@@ -119,13 +119,14 @@ struct ot_batch_s {
   bool own_main = false;
   cudaEvent_t fork = nullptr, t0 = nullptr, t1 = nullptr;
   std::vector<cudaEvent_t> join;
-  cudaGraphExec_t gexec[2] = {nullptr, nullptr};
+  cudaGraphExec_t gexec[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};   // [parity][0: a pair, 1: kBatchLong pairs]
   ~ot_batch_s() {
     if (main) cudaStreamSynchronize(main);
     for (auto& g : groups)
       if (g && g->st) cudaStreamSynchronize(g->st);
-    for (auto& e : gexec)
-      if (e) cudaGraphExecDestroy(e);
+    for (auto& row : gexec)
+      for (auto& e : row)
+        if (e) cudaGraphExecDestroy(e);
     for (cudaEvent_t e : {fork, t0, t1})
       if (e) cudaEventDestroy(e);
     for (cudaEvent_t e : join)
@@ -147,22 +148,24 @@ bool same_shape(const ot_grid& a, const ot_grid& b) {
 
 ot_status make_plan(const ot_grid& g, int batch, void* stream, std::unique_ptr<PlanBase>& out);
 
-// fork from the main stream to every group stream and join back
-ot_status batch_capture(ot_batch_s& b, int parity) {
-  if (b.gexec[parity]) return OT_OK;
+// fork from the main stream to every group stream, a pair of iterations (or kBatchLong pairs) per group, and join back
+constexpr int kBatchLong = 4;
+ot_status batch_capture(ot_batch_s& b, int parity, int pairs) {
+  cudaGraphExec_t& ge = b.gexec[parity][pairs > 1];
+  if (ge) return OT_OK;
   cudaGraph_t gr = nullptr;
   CUDA_OK(cudaStreamBeginCapture(b.main, cudaStreamCaptureModeThreadLocal));
   CUDA_OK(cudaEventRecord(b.fork, b.main));
   for (size_t i = 0; i < b.groups.size(); ++i) {
     PlanBase& P = *b.groups[i];
     CUDA_OK(cudaStreamWaitEvent(P.st, b.fork, 0));
-    OT_TRY(P.enqueue_pair());
+    for (int k = 0; k < pairs; ++k) OT_TRY(P.enqueue_pair());
     CUDA_OK(cudaEventRecord(b.join[i], P.st));
     CUDA_OK(cudaStreamWaitEvent(b.main, b.join[i], 0));
   }
   cudaError_t e = cudaStreamEndCapture(b.main, &gr);
   if (e != cudaSuccess) return seterr(OT_ECUDA, "batch graph capture: %s", cudaGetErrorString(e));
-  e = cudaGraphInstantiate(&b.gexec[parity], gr, 0);
+  e = cudaGraphInstantiate(&ge, gr, 0);
   cudaGraphDestroy(gr);
   if (e != cudaSuccess) return seterr(OT_ECUDA, "batch graph instantiate: %s", cudaGetErrorString(e));
   return OT_OK;
@@ -318,8 +321,12 @@ ot_status ot_batch_solve(ot_batch_t b, const float* const* f0, const float* cons
       const int chunk = std::min(K, iters - done);
       const int plain = chunk - 1;
       const int par = b->groups[0]->parity();
-      if (plain >= 2) OT_TRY(batch_capture(*b, par));
-      for (int r = 0; r < plain / 2; ++r) CUDA_OK(cudaGraphLaunch(b->gexec[par], b->main));
+      for (int r = plain / 2; r > 0;) {
+        const int pairs = r >= kBatchLong ? kBatchLong : 1;
+        OT_TRY(batch_capture(*b, par, pairs));
+        CUDA_OK(cudaGraphLaunch(b->gexec[par][pairs > 1], b->main));
+        r -= pairs;
+      }
       // the remaining single iteration and the checked one, per group after the graph
       CUDA_OK(cudaEventRecord(b->fork, b->main));
       for (size_t i = 0; i < b->groups.size(); ++i) {

@@ -154,7 +154,7 @@ struct Plan final : PlanBase {
   int tc = 0;               // time-chunk length of the tiled update (autotuned)
   int par = 0;              // buffer holding the current state
   bool have_x = false;
-  cudaGraphExec_t gexec[2] = {nullptr, nullptr};
+  cudaGraphExec_t gexec[2] = {nullptr, nullptr}, glong[2] = {nullptr, nullptr};   // 2 and kLongGraph iterations
   // [parity][lead]: the check iteration (x written) with its reductions and the copies of the results
   // to pinned host memory, optionally preceded by one plain iteration
   cudaGraphExec_t gcheck[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
@@ -162,6 +162,8 @@ struct Plan final : PlanBase {
 
   ~Plan() override {
     for (auto& e : gexec)
+      if (e) cudaGraphExecDestroy(e);
+    for (auto& e : glong)
       if (e) cudaGraphExecDestroy(e);
     for (auto& row : gcheck)
       for (auto& e : row)
@@ -981,12 +983,13 @@ struct Plan final : PlanBase {
     if (evs) cudaEventRecord(evs[4], st);
   }
 
-  ot_status graph_for(int p) {
-    if (gexec[p]) return OT_OK;
+  // `iters` (even) plain iterations from buffer p as one graph
+  ot_status graph_for(int p, int iters = 2) {
+    cudaGraphExec_t& ge = iters == 2 ? gexec[p] : glong[p];
+    if (ge) return OT_OK;
     cudaGraph_t gr = nullptr;
     CUDA_OK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-    enqueue_iteration(p, false, false);
-    enqueue_iteration(1 - p, false, false);
+    for (int i = 0; i < iters; ++i) enqueue_iteration(p ^ (i & 1), false, false);
     const cudaError_t le = cudaGetLastError();
     cudaError_t e = cudaStreamEndCapture(st, &gr);
     if (le != cudaSuccess) {
@@ -994,18 +997,20 @@ struct Plan final : PlanBase {
       return seterr(OT_ECUDA, "kernel launch during graph capture: %s", cudaGetErrorString(le));
     }
     if (e != cudaSuccess) return seterr(OT_ECUDA, "graph capture: %s", cudaGetErrorString(e));
-    e = cudaGraphInstantiate(&gexec[p], gr, 0);
+    e = cudaGraphInstantiate(&ge, gr, 0);
     cudaGraphDestroy(gr);
     if (e != cudaSuccess) return seterr(OT_ECUDA, "graph instantiate: %s", cudaGetErrorString(e));
     return OT_OK;
   }
 
-  // plain iterations (no residual, no x output), pairs from a graph
+  // plain iterations (no residual, no x output): graphs of kLongGraph iterations, then of pairs
+  static constexpr int kLongGraph = 8;
   ot_status run_plain(int n) {
     while (n >= 2) {
-      OT_TRY(graph_for(par));
-      CUDA_OK(cudaGraphLaunch(gexec[par], st));
-      n -= 2;
+      const int k = n >= kLongGraph ? kLongGraph : 2;
+      OT_TRY(graph_for(par, k));
+      CUDA_OK(cudaGraphLaunch(k == 2 ? gexec[par] : glong[par], st));
+      n -= k;
     }
     if (n == 1) {
       enqueue_iteration(par, false, false);
@@ -1310,7 +1315,7 @@ struct Plan final : PlanBase {
   int parity() const override { return par; }
 
   ot_status enable_retirement() override {
-    if (gexec[0] || gexec[1]) return seterr(OT_EINVAL, "retirement must be enabled before graphs are captured");
+    if (gexec[0] || gexec[1] || glong[0] || glong[1]) return seterr(OT_EINVAL, "retirement must be enabled before graphs are captured");
     h_active.assign(B, 1);
     CUDA_OK(cudaMemcpyAsync(active, h_active.data(), sizeof(int) * B, cudaMemcpyHostToDevice, st));
     CUDA_OK(cudaStreamSynchronize(st));
