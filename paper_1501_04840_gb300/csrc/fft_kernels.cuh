@@ -142,14 +142,6 @@ inline size_t fft_yc_smem(int m1, int m2, int C) {
          sizeof(double) * (n + fft_yc_w(C));
 }
 
-// a / b in double to about 2^-40 (the quotient of a low mode is rounded to FP32): the approximate reciprocal and one
-// Newton step, a quarter of a division's instructions on the FP64 pipe.  The blocks that hold the low modes are the last
-// to finish.
-__device__ __forceinline__ double quot_low(double a, double b) {
-  const double r = rcp_approx(b);
-  return a * fma(fma(-b, r, 1.0), r, r);
-}
-
 template <typename T, int M1, int M2, int C>
 __global__ void __launch_bounds__(kFftNP* M1, M2 >= 32 ? 2 : 768 / (kFftNP * M1))
     k_fft_yc(Geo<T> g, T* __restrict__ hat, YcTables tb) {

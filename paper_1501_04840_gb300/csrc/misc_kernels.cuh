@@ -123,27 +123,51 @@ __global__ void k_unpack_path(Geo<T> g, Compact cp, const float* __restrict__ pa
   }
 }
 
-// packed (float, times scale) <- internal; dst[k] may be separate arrays (stride per problem lenk)
+// v times scale, rounded to FP32 once: for FP32 values the product's error and the scale's remainder are carried in a
+// second FP32 value (an FP64 product and two conversions per value took 140 us for a path of 25 M values).
 template <typename T>
-__global__ void k_pack_path(Geo<T> g, Compact cp, const v4<T>* xi, double scale,
-                            float* __restrict__ packed, float* d0, float* d1, float* d2, float* d3) {
-  const long long tot = (long long)g.B * g.N;
-  float* ds[4] = {d0, d1, d2, d3};
-  for (long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x; id < tot; id += (long long)gridDim.x * blockDim.x) {
-    long long r = id;
-    const int x = r % g.n1; r /= g.n1;
-    const int y = r % g.n2; r /= g.n2;
-    const int c = r % g.C; r /= g.C;
-    const int t = r % g.P;
-    const int b = (int)(r / g.P);
+__device__ __forceinline__ float scaled(T v, double scale, float sh, float sl) {
+  if constexpr (sizeof(T) == 4) {
+    if (sh == 0.f) return (float)((double)v * scale);
+    const float p = v * sh;
+    return p + fmaf(v, sl, fmaf(v, sh, -p));
+  } else {
+    return (float)((double)v * scale);
+  }
+}
+
+// packed (float, times scale) <- internal, problem blockIdx.y; scales[problem], or none (nullptr); d0..d3: the components
+// as separate arrays [problem][len_k].  Cells are indexed in 32 bits inside a problem.
+template <typename T>
+__global__ void __launch_bounds__(256) k_pack_path(Geo<T> g, Compact cp, const v4<T>* __restrict__ xi,
+                                                   const double* __restrict__ scales, float* __restrict__ packed,
+                                                   float* d0, float* d1, float* d2, float* d3) {
+  const int b = blockIdx.y;
+  const double scale = scales ? scales[b] : 1.0;
+  // the two-value product where neither it nor its parts can leave FP32's normal range by the scale alone
+  const bool split = scale > 1e-18 && scale < 1e18;
+  const float sh = split ? (float)scale : 0.f, sl = split ? (float)(scale - (double)sh) : 0.f;
+  float* ds[4];
+  float* in[4] = {d0, d1, d2, d3};
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const long long ci = cp.index(k, t, x, y, c);
-      if (ci < 0) continue;
-      const float v = (float)((double)comp<T>(xi, id, k) * scale);
-      if (packed) packed[(long long)b * cp.total + ci] = v;
-      if (ds[k]) ds[k][(long long)b * cp.len[k] + ci - cp.off[k]] = v;
+  for (int k = 0; k < 4; ++k)
+    ds[k] = packed ? packed + (long long)b * cp.total + cp.off[k] : (in[k] ? in[k] + (long long)b * cp.len[k] : nullptr);
+  const unsigned n1 = g.n1, n2 = g.n2, C = g.C, N = (unsigned)g.N;
+  const v4<T>* src = xi + (size_t)b * N;
+  for (unsigned id = blockIdx.x * 256 + threadIdx.x; id < N; id += gridDim.x * 256) {
+    const unsigned rx = id / n1, x = id - rx * n1, ry = rx / n2, y = rx - ry * n2, t = ry / C, c = ry - t * C;
+    const v4<T> v = src[id];
+    const unsigned i[3] = {x, y, c}, n[3] = {n1, n2, C};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      if (k >= cp.d || !ds[k]) continue;
+      unsigned j[3] = {i[0], i[1], i[2]}, m[3] = {n[0], n[1], n[2]};
+      if (cp.per[k]) j[k] = i[k] + 1 == n[k] ? 0 : i[k] + 1;   // internal face right of cell i = paper face i + 1
+      else if (i[k] + 1 == n[k]) continue;                      // the absent boundary face
+      else m[k] = n[k] - 1;
+      ds[k][j[0] + m[0] * (j[1] + m[1] * (j[2] + m[2] * t))] = scaled<T>(cget<T>(v, k), scale, sh, sl);
     }
+    if (ds[3] && t + 1 < (unsigned)g.P) ds[3][id] = scaled<T>(v.w, scale, sh, sl);
   }
 }
 
@@ -226,28 +250,31 @@ __global__ void k_dual_init(Geo<T> g, const v4<T>* __restrict__ x, const T* __re
 }
 
 // w = K x0 + (0, f_b^+) at the cells (S_M m0 and S_F f0 + f_b^+ of section 2) for the least-norm feasible
-// path x0 = (m0, f0): the dual value of a check is sigma <b, w> (the dual function of the problem at
-// p = sigma b, with the infimum over C_d taken at x0).
+// path x0 = -A^T phi, problem blockIdx.y: the dual value of a check is sigma <b, w> (the dual function of the problem at
+// p = sigma b, with the infimum over C_d taken at x0).  The faces of x0 are differences of phi and are formed in place.
 template <typename T>
-__global__ void k_dual_weights(Geo<T> g, const v4<T>* __restrict__ x, const T* __restrict__ f0,
-                               const T* __restrict__ f1, v4<T>* __restrict__ w) {
-  const long long tot = (long long)g.B * g.N;
-  for (long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x; id < tot; id += (long long)gridDim.x * blockDim.x) {
-    long long r = id;
-    const int ix = r % g.n1; r /= g.n1;
-    const int iy = r % g.n2; r /= g.n2;
-    const int ic = r % g.C; r /= g.C;
-    const int t = r % g.P;
-    const int b = (int)(r / g.P);
-    T left[3];
-    left[0] = ix > 0 ? comp<T>(x, cidx(g, b, t, ix - 1, iy, ic), 0) : (g.per1 ? comp<T>(x, cidx(g, b, t, g.n1 - 1, iy, ic), 0) : T(0));
-    left[1] = iy > 0 ? comp<T>(x, cidx(g, b, t, ix, iy - 1, ic), 1) : (g.per2 ? comp<T>(x, cidx(g, b, t, ix, g.n2 - 1, ic), 1) : T(0));
-    left[2] = ic > 0 ? comp<T>(x, cidx(g, b, t, ix, iy, ic - 1), 2) : (g.perc ? comp<T>(x, cidx(g, b, t, ix, iy, g.C - 1), 2) : T(0));
-    const size_t s = (size_t)b * g.S + ix + (size_t)g.n1 * (iy + (size_t)g.n2 * ic);
-    const T fl = t == 0 ? f0[s] : comp<T>(x, cidx(g, b, t - 1, ix, iy, ic), 3);
-    const T fr = t == g.P - 1 ? f1[s] : comp<T>(x, id, 3);
-    w[id] = mk4<T>(T(0.5) * (left[0] + comp<T>(x, id, 0)), T(0.5) * (left[1] + comp<T>(x, id, 1)),
-                   T(0.5) * (left[2] + comp<T>(x, id, 2)), T(0.5) * (fl + fr));
+__global__ void __launch_bounds__(256) k_dual_weights(Geo<T> g, const T* __restrict__ phi, const T* __restrict__ f0,
+                                                      const T* __restrict__ f1, v4<T>* __restrict__ w) {
+  const int b = blockIdx.y;
+  const unsigned n1 = g.n1, n2 = g.n2, C = g.C, P = g.P, N = (unsigned)g.N, S = g.S;
+  const T* ph = phi + (size_t)b * N;
+  const T *p0 = f0 + (size_t)b * S, *p1 = f1 + (size_t)b * S;
+  v4<T>* out = w + (size_t)b * N;
+  for (unsigned id = blockIdx.x * 256 + threadIdx.x; id < N; id += gridDim.x * 256) {
+    const unsigned rx = id / n1, x = id - rx * n1, ry = rx / n2, y = rx - ry * n2, t = ry / C, c = ry - t * C;
+    const T v = ph[id];
+    // faces left and right of the cell along one axis: s (phi_next - phi), zero where a Neumann axis ends
+    auto both = [&](unsigned i, unsigned n, unsigned stride, int per, T s) {
+      const bool first = i == 0, last = i + 1 == n;
+      const T left = first && !per ? T(0) : s * (v - ph[first ? id + (n - 1) * stride : id - stride]);
+      const T right = last && !per ? T(0) : s * (ph[last ? id - (n - 1) * stride : id + stride] - v);
+      return T(0.5) * (left + right);
+    };
+    const unsigned cell = id - t * S;
+    const T lo = t == 0 ? p0[cell] : g.sp * (v - ph[id - S]);
+    const T hi = t + 1 == P ? p1[cell] : g.sp * (ph[id + S] - v);
+    out[id] = mk4<T>(both(x, n1, 1, g.per1, g.s1), both(y, n2, n1, g.per2, g.s2), both(c, C, n1 * n2, g.perc, g.sc),
+                     T(0.5) * (lo + hi));
   }
 }
 

@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(kMmXtThreads, sizeof(T) == 4 ? 2 : 1)
     const v4<T>* pc = ap + rowbase;
     const T* pf0 = f0 + (size_t)b * S + (rowbase - (size_t)b * P * S);
     const T* pf1 = f1 + (size_t)b * S + (rowbase - (size_t)b * P * S);
-    // four cells of the row-major plane per thread and pass, all their loads in flight together
+    // four cells of the row-major plane per thread and pass, all their loads in flight together (eight were slower)
     constexpr int U = 4;
     const int total = P * n1, dt = blockDim.x / n1, dxs = blockDim.x - dt * n1;
     int t = threadIdx.x / n1, x = threadIdx.x - t * n1;
@@ -425,7 +425,9 @@ inline int mm_yc_wt(int C) { return C == 1 ? 8 : (C == 4 ? 2 : 4); }
 inline int mm_yc_ld(int C, int W) { return (C * W + 7) / 8 * 8 + 4; }
 constexpr int kMmYcThreads = 256;
 template <typename T>
-inline size_t mm_yc_smem(int n2, int C, int W, int buf) { return sizeof(T) * ((size_t)n2 * mm_yc_ld(C, W) + buf); }
+inline size_t mm_yc_smem(int n2, int C, int W, int buf) {
+  return sizeof(T) * ((size_t)n2 * mm_yc_ld(C, W) + buf + n2 + W) + 8 + sizeof(double) * (n2 + W);
+}
 inline int mm_yc_items(int lf, int C, int W) { return (W / mm_yc_wt(C)) * (lf / 4); }
 
 template <typename T, int C>
@@ -447,6 +449,19 @@ __global__ void __launch_bounds__(kMmYcThreads, sizeof(T) == 4 ? 2 : 1) k_mm_yc(
     for (int j = 0; j < C; ++j) Q[c][j] = ((const T*)tb.Qc)[c * C + j];
   }
   const T lt = ((const T*)tb.lamt)[kt];
+  const double ltd = tb.lamtd[kt];
+  T* l2 = buf + mm_buf(ay.l0, ay.lf, ay.li);   // eigenvalues along y and x (the strip), also in double
+  T* l1 = l2 + n2;
+  double* l2d = (double*)(((uintptr_t)(l1 + W) + 7) & ~uintptr_t(7));
+  double* l1d = l2d + n2;
+  for (int j = threadIdx.x; j < n2; j += blockDim.x) {
+    l2[j] = ((const T*)tb.lam2)[j];
+    l2d[j] = tb.lam2d[j];
+  }
+  if ((int)threadIdx.x < W) {
+    l1[threadIdx.x] = ((const T*)tb.lam1)[min(x0 + (int)threadIdx.x, n1 - 1)];
+    l1d[threadIdx.x] = tb.lam1d[min(x0 + (int)threadIdx.x, n1 - 1)];
+  }
   pdl_wait();   // the spectral array (forward x/t pass) is read from here on
   const size_t plane = ((size_t)b * g.P + kt) * g.S + x0;
   constexpr int V = sizeof(T) == 4 ? 4 : 2;
@@ -503,7 +518,7 @@ __global__ void __launch_bounds__(kMmYcThreads, sizeof(T) == 4 ? 2 : 1) k_mm_yc(
       T r[C], co[C];
 #pragma unroll
       for (int cc = 0; cc < C; ++cc) r[cc] = p[cc * WT];
-      const T lxyt = ((const T*)tb.lam1)[x0 + w] + ((const T*)tb.lam2)[ky] + lt;
+      const T lxyt = l1[w] + l2[ky] + lt;
 #pragma unroll
       for (int j = 0; j < C; ++j) {
         T s = 0;
@@ -514,8 +529,8 @@ __global__ void __launch_bounds__(kMmYcThreads, sizeof(T) == 4 ? 2 : 1) k_mm_yc(
           co[j] = T(0);     // the zero eigenvalue of the pseudo-inverse
         } else if ((float)lam < thr) {
           // low modes: eigenvalue and quotient in double precision
-          const double ld_ = tb.lam1d[x0 + w] + tb.lam2d[ky] + tb.lamtd[kt] + tb.lamcd[j];
-          co[j] = ld_ > 0.0 ? (T)((double)s / ld_) : T(0);
+          const double ld_ = l1d[w] + l2d[ky] + ltd + tb.lamcd[j];
+          co[j] = ld_ > 0.0 ? (T)quot_low((double)s, ld_) : T(0);
         } else {
           co[j] = fdiv_fast(s, lam);
         }

@@ -92,7 +92,7 @@ struct Plan final : PlanBase {
   double* acc = nullptr;    // [B][kAcc]
   double* mass = nullptr;   // [B][P]
   double* chk = nullptr;    // [B][kChk]
-  double* scl = nullptr;    // [B][2]
+  double* scl = nullptr;    // [B][2] densities -> solver units, then [B] solver -> caller units (out_scale)
   double* part = nullptr;   // per-block partial sums of the residual check
   int* err = nullptr;       // set by a kernel whose bounded device wait ran out (sticky until the next start)
   int* active = nullptr;    // [B] per-problem flags of a retiring batch (g.active points here once enabled)
@@ -207,7 +207,7 @@ struct Plan final : PlanBase {
     size_t bytes = narr * rnd16(cells * sizeof(T)) + 2 * rnd16((size_t)B * S * sizeof(T)) +
                    rnd16(stage_floats * sizeof(float)) + rnd16(sizeof(double) * B * kAcc) +
                    rnd16(sizeof(double) * (size_t)B * P) + rnd16(sizeof(double) * B * kChk) +
-                   rnd16(sizeof(double) * B * 2) + rnd16(part_bytes()) + 16 + rnd16(sizeof(int) * B);
+                   rnd16(sizeof(double) * B * 3) + rnd16(part_bytes()) + 16 + rnd16(sizeof(int) * B);
     CUDA_OK(cudaMalloc(&mem.p, bytes));
     char* q = (char*)mem.p;
     auto take = [&](size_t nb) { char* r = q; q += rnd16(nb); return r; };
@@ -224,7 +224,7 @@ struct Plan final : PlanBase {
     mass = (double*)take(sizeof(double) * (size_t)B * P);
     err = (int*)take(sizeof(int));
     chk = (double*)take(sizeof(double) * B * kChk);
-    scl = (double*)take(sizeof(double) * B * 2);
+    scl = (double*)take(sizeof(double) * B * 3);
     part = (double*)take(part_bytes());
     active = (int*)take(sizeof(int) * B);
     CUDA_OK(cudaMemsetAsync(mem.p, 0, bytes, st));
@@ -303,7 +303,7 @@ struct Plan final : PlanBase {
 
   // Autotuner, run once per shape and device (the choice is cached for later plans of the shape):
   //  - the tiled update: staged by bulk tensor copies or with plain loads (where both exist), and time chunks
-  //    of P, P/2, P/4 or P/8 planes, each timed over whole iterations (FP32).
+  //    of P, P/2, P/4 or P/8 planes (3 and 2 on small grids), each timed over whole iterations (FP32).
   // Each candidate is timed over ten launches (after two untimed ones) on the zeroed workspace (b set so that the prox takes its
   // Newton branch); a later candidate must beat the best by 3 % (1 % for the FP32 update, timed over whole iterations,
   // where the update's share dilutes its differences; ties keep the earlier, simpler one).
@@ -349,6 +349,12 @@ struct Plan final : PlanBase {
       if (c >= 4 || d == 1)
         if (std::find(cands.begin(), cands.end(), c) == cands.end()) cands.push_back(c);
     }
+    // small grids: a block's planes follow one another, so shorter chunks on idle SMs pay for the plane they recompute
+    if (tiled)
+      for (int c : {3, 2}) {
+        const dim3 gr = tiled_grid(c);
+        if (c < cands.back() && (long long)gr.x * gr.y * gr.z <= 8 * 152) cands.push_back(c);
+      }
     tc = cands[0];
     use_tma = tma_ok;
     const std::string key = shape_key();
@@ -1176,7 +1182,7 @@ struct Plan final : PlanBase {
   // validate the staged densities (section 2: f >= 0, equal masses) and rescale (reading of section 4)
   ot_status validate_scale(bool normalise) {
     const size_t n = (size_t)B * S;
-    std::vector<double> sc(2 * B, 1.0);
+    std::vector<double> sc(3 * B, 1.0);
     if (normalise) {
       CUDA_OK(cudaMemsetAsync(chk, 0, sizeof(double) * B * kChk, st));
       // minima start at +inf
@@ -1203,6 +1209,7 @@ struct Plan final : PlanBase {
     } else {
       for (int bi = 0; bi < B; ++bi) out_scale[bi] = 1.0;
     }
+    for (int bi = 0; bi < B; ++bi) sc[2 * B + bi] = out_scale[bi];
     CUDA_OK(cudaMemcpyAsync(scl, sc.data(), sc.size() * sizeof(double), cudaMemcpyHostToDevice, st));
     const int blocks = std::min(1024, (S + 255) / 256);
     k_scale_boundary<T><<<dim3(blocks, B), 256, 0, st>>>(stage, stage + n, S, scl, f0n, f1n);
@@ -1222,19 +1229,10 @@ struct Plan final : PlanBase {
   }
 
   // w = K x0 + (0, f_b^+) for the boundary densities in f0n, f1n, with x0 = Pi_{C_d}(0) the least-norm feasible
-  // path (the projection of step 1 applied to a = 0); x serves as the work array.
+  // path (the projection of step 1 applied to a = 0, which a[0] holds).
   ot_status make_dual_weights() {
-    const long long cells = (long long)B * N;
-    CUDA_OK(cudaMemsetAsync(x, 0, cells * sizeof(v4<T>), st));
-    enqueue_poisson_src(x, nullptr);
-    Arrays<T> A{};
-    A.a = x;
-    A.x = x;   // in place: every cell reads only its own a
-    A.phi = phi;
-    A.f0 = f0n;
-    A.f1 = f1n;
-    k_correct<T><<<grid1d(cells), 256, 0, st>>>(g, A);
-    k_dual_weights<T><<<grid1d(cells), 256, 0, st>>>(g, x, f0n, f1n, w);
+    enqueue_poisson(0, nullptr);
+    k_dual_weights<T><<<dim3(grid1d(N), B), 256, 0, st>>>(g, phi, f0n, f1n, w);
     CUDA_OK(cudaGetLastError());
     have_x = false;
     return OT_OK;
@@ -1341,8 +1339,8 @@ struct Plan final : PlanBase {
       if (!ds[k]) continue;
       float* dd[4] = {nullptr, nullptr, nullptr, nullptr};
       dd[k] = stage;
-      k_pack_path<T><<<grid1d(N), 256, 0, st>>>(g1, cp, x + off, out_scale[bi], nullptr, dd[0], dd[1], dd[2],
-                                                dd[3]);
+      k_pack_path<T><<<dim3(grid1d(N), 1), 256, 0, st>>>(g1, cp, x + off, scl + 2 * B + bi, nullptr, dd[0], dd[1],
+                                                         dd[2], dd[3]);
       CUDA_OK(cudaGetLastError());
       CUDA_OK(cudaMemcpyAsync(ds[k], stage, (size_t)cp.len[k] * sizeof(float), cudaMemcpyDefault, st));
       CUDA_OK(cudaStreamSynchronize(st));
@@ -1356,16 +1354,10 @@ struct Plan final : PlanBase {
     for (int k = 0; k < 4; ++k) {
       if (!ds[k]) continue;
       // component k of every problem, scaled back to the caller's units
-      for (int bi = 0; bi < B; ++bi) {
-        Geo<T> g1 = g;
-        g1.B = 1;
-        const size_t off = (size_t)bi * N;
-        float* dd[4] = {nullptr, nullptr, nullptr, nullptr};
-        dd[k] = stage + (size_t)bi * cp.len[k];
-        k_pack_path<T><<<grid1d(N), 256, 0, st>>>(g1, cp, x + off, out_scale[bi], nullptr, dd[0], dd[1], dd[2],
-                                                  dd[3]);
-        CUDA_OK(cudaGetLastError());
-      }
+      float* dd[4] = {nullptr, nullptr, nullptr, nullptr};
+      dd[k] = stage;
+      k_pack_path<T><<<dim3(grid1d(N), B), 256, 0, st>>>(g, cp, x, scl + 2 * B, nullptr, dd[0], dd[1], dd[2], dd[3]);
+      CUDA_OK(cudaGetLastError());
       CUDA_OK(cudaMemcpyAsync(ds[k], stage, (size_t)B * cp.len[k] * sizeof(float), cudaMemcpyDefault, st));
       CUDA_OK(cudaStreamSynchronize(st));
     }
@@ -1376,9 +1368,10 @@ struct Plan final : PlanBase {
                       const float* bbp) override {
     if (!f0 || !f1 || !xp || !bp) return seterr(OT_EINVAL, "f0, f1, x and b are required");
     OT_TRY(load_boundary(f0, f1, false));
+    const long long cells = (long long)B * N;
+    CUDA_OK(cudaMemsetAsync(a[0], 0, cells * sizeof(v4<T>), st));
     OT_TRY(make_dual_weights());
     OT_TRY(unpack_x(xp));
-    const long long cells = (long long)B * N;
     CUDA_OK(cudaMemsetAsync(err, 0, sizeof(int), st));
     *h_err = 0;
     // b -> b[0]; bbar -> b[1] temporarily
@@ -1426,7 +1419,7 @@ struct Plan final : PlanBase {
     const long long cells = (long long)B * N;
     if (xp) {
       if (!have_x) return seterr(OT_EINVAL, "x is not available: run ot_iterate first");
-      k_pack_path<T><<<grid1d(cells), 256, 0, st>>>(g, cp, x, 1.0, stage, nullptr, nullptr, nullptr, nullptr);
+      k_pack_path<T><<<dim3(grid1d(N), B), 256, 0, st>>>(g, cp, x, nullptr, stage, nullptr, nullptr, nullptr, nullptr);
       CUDA_OK(cudaGetLastError());
       CUDA_OK(cudaMemcpyAsync(xp, stage, (size_t)B * cp.total * sizeof(float), cudaMemcpyDefault, st));
       CUDA_OK(cudaStreamSynchronize(st));
@@ -1467,7 +1460,7 @@ struct Plan final : PlanBase {
     Arrays<T> A = arrays(0, true);
     k_correct<T><<<grid1d(cells), 256, 0, st>>>(g, A);
     CUDA_OK(cudaGetLastError());
-    k_pack_path<T><<<grid1d(cells), 256, 0, st>>>(g, cp, x, 1.0, stage, nullptr, nullptr, nullptr, nullptr);
+    k_pack_path<T><<<dim3(grid1d(N), B), 256, 0, st>>>(g, cp, x, nullptr, stage, nullptr, nullptr, nullptr, nullptr);
     CUDA_OK(cudaGetLastError());
     CUDA_OK(cudaMemcpyAsync(xp, stage, (size_t)B * cp.total * sizeof(float), cudaMemcpyDefault, st));
     if (phip) {

@@ -71,6 +71,14 @@ __device__ __forceinline__ double rcp_approx(double x) {
   return r;
 }
 
+// a / b in double to about 2^-40 (the quotient of a low mode is rounded to FP32): the approximate reciprocal and one
+// Newton step, a quarter of a division's instructions on the FP64 pipe.  The blocks that hold the low modes are the last
+// to finish.
+__device__ __forceinline__ double quot_low(double a, double b) {
+  const double r = rcp_approx(b);
+  return a * fma(fma(-b, r, 1.0), r, r);
+}
+
 // The root of q(z) = (1 + z)^2 (z - e) - d in FP64 (e + d > 0; |e| and d far from overflow).  The FP64 pipe is a
 // sixty-fourth of the FP32 one, so the start comes from FP32: bound and three Newton steps as prox_J<float> takes
 // them, good to about 1e-7 of |e| + d + z.  From there Newton converges quadratically from either side (q is
