@@ -408,16 +408,24 @@ __global__ void __launch_bounds__(128) k_conv3d_wgrad_tiled(Vol v, int Cin, int 
 }
 
 // dw[co][tap][ci] += sum over the blocks of one channel slice of their partials
-__global__ void k_wgrad_reduce(int Cin, int nblk, const float* __restrict__ part, float* __restrict__ dw) {
-  const int slice = blockIdx.y, nci = Cin / 16;
-  const int ci0 = (slice % nci) * 16, co0 = (slice / nci) * 16;
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < 27 * 256; e += gridDim.x * blockDim.x) {
-    const float* p = part + (size_t)slice * nblk * (27 * 256) + e;
-    float s = 0.f;
-    for (int k = 0; k < nblk; ++k) s += p[(size_t)k * (27 * 256)];
-    const int tap = e / 256, co = (e / 16) % 16, ci = e % 16;
-    dw[((size_t)(co0 + co) * 27 + tap) * Cin + ci0 + ci] += s;
-  }
+// (32 consecutive values per block, the partials in eight interleaved runs, one per warp, added in order: one thread per
+// value walked 608 partials one after another, 57 us for 6912 values)
+__global__ void __launch_bounds__(256) k_wgrad_reduce(int Cin, int nblk, const float* __restrict__ part,
+                                                      float* __restrict__ dw) {
+  const int slice = blockIdx.y, nci = Cin / 16, lane = threadIdx.x & 31, run = threadIdx.x >> 5;
+  const int ci0 = (slice % nci) * 16, co0 = (slice / nci) * 16, e = blockIdx.x * 32 + lane;
+  const float* p = part + (size_t)slice * nblk * (27 * 256) + e;
+  float s = 0.f;
+#pragma unroll 8
+  for (int k = run; k < nblk; k += 8) s += p[(size_t)k * (27 * 256)];
+  __shared__ float red[8][32];
+  red[run][lane] = s;
+  __syncthreads();
+  if (run) return;
+#pragma unroll
+  for (int r = 1; r < 8; ++r) s += red[r][lane];
+  const int tap = e / 256, co = (e / 16) % 16, ci = e % 16;
+  dw[((size_t)(co0 + co) * 27 + tap) * Cin + ci0 + ci] += s;
 }
 
 // dw[co][tap][ci] += sum over the chunks of the tcgen05 weight gradient's partials [chunk][tap][co][ci]
@@ -433,6 +441,38 @@ __global__ void k_wgrad_reduce_tc(int Cin, int Cout, int nchunks, const float* _
 }
 
 // db[c] += sum_v dy[v][c]
+// db[c] += sum of dy's channel c, eight channels (16 bytes) per thread: the tensor is read once, where a block per
+// channel read two bytes out of every voxel (50 against 15 us for 2.1 M voxels of 16 channels).
+__global__ void __launch_bounds__(256) k_bias_grad_vec(long long M, int C, const bf16* __restrict__ dy, int dys, int dyo,
+                                                       float* __restrict__ db) {
+  const int groups = C / 8, per = 256 / groups;   // voxels per pass of the block
+  const int cg = threadIdx.x % groups, v0 = threadIdx.x / groups;
+  float acc[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) acc[q] = 0.f;
+  if (v0 < per) {
+#pragma unroll 4
+    for (long long v = (long long)blockIdx.x * per + v0; v < M; v += (long long)gridDim.x * per) {
+      const uint4 r = *reinterpret_cast<const uint4*>(dy + v * dys + dyo + 8 * cg);
+      const uint32_t w[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        acc[2 * q] += __uint_as_float(w[q] << 16);
+        acc[2 * q + 1] += __uint_as_float(w[q] & 0xffff0000u);
+      }
+    }
+  }
+  __shared__ float red[256][9];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) red[threadIdx.x][q] = acc[q];
+  __syncthreads();
+  if ((int)threadIdx.x < C) {
+    const int g = threadIdx.x / 8, q = threadIdx.x % 8;
+    float t = 0.f;
+    for (int v = 0; v < per; ++v) t += red[v * groups + g][q];
+    atomicAdd(&db[threadIdx.x], t);
+  }
+}
 __global__ void k_bias_grad(long long M, int C, const bf16* __restrict__ dy, int dys, int dyo, float* __restrict__ db) {
   const int c = blockIdx.y;
   float s = 0.f;
@@ -462,6 +502,28 @@ __global__ void k_rotate_weights(int Cin, int Cout, const bf16* __restrict__ w, 
 }
 
 // g[v][c] *= (y[v][c] > 0)  (ReLU backward on the stored activation)
+// g *= (y > 0), eight channels (16 bytes) per thread: 86 -> 35 us for 2.1 M voxels of 16 channels.
+__global__ void __launch_bounds__(256) k_relu_grad_vec(long long M, int groups, bf16* __restrict__ g, int gs, int go,
+                                                       const bf16* __restrict__ y, int ys, int yo) {
+  const long long n = M * groups;
+#pragma unroll 2
+  for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n; i += gridDim.x * 256ll) {
+    const long long vv = n < (1ll << 32) ? (long long)((unsigned)i / (unsigned)groups) : i / groups;
+    const int c = 8 * (int)(i - vv * groups);
+    const uint4 r = *reinterpret_cast<const uint4*>(y + vv * ys + yo + c);
+    uint4* gp = reinterpret_cast<uint4*>(g + vv * gs + go + c);
+    const uint4 u = *gp;
+    const uint32_t w[4] = {r.x, r.y, r.z, r.w}, d[4] = {u.x, u.y, u.z, u.w};
+    uint32_t o[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const uint32_t lo = __uint_as_float(w[q] << 16) > 0.f ? 0xffffu : 0u;
+      const uint32_t hi = __uint_as_float(w[q] & 0xffff0000u) > 0.f ? 0xffff0000u : 0u;
+      o[q] = d[q] & (lo | hi);
+    }
+    *gp = make_uint4(o[0], o[1], o[2], o[3]);
+  }
+}
 __global__ void k_relu_grad(long long M, int C, bf16* __restrict__ g, int gs, int go, const bf16* __restrict__ y,
                             int ys, int yo) {
   const long long n = M * C;
@@ -674,6 +736,14 @@ __global__ void k_dual_channels(int Y, int X, int P, int to_channels, float* __r
 }
 
 inline int blocks_for(long long n) { return (int)((n + 255) / 256 < 152 * 32 ? (n + 255) / 256 : 152 * 32); }
+
+// 16-byte pieces where the slice allows them and a block holds every channel; otherwise a block row per channel
+inline void launch_bias_grad(long long M, int C, const bf16* dy, int dys, int dyo, float* db, cudaStream_t st) {
+  if (C % 8 == 0 && C <= 256 && dys % 8 == 0 && dyo % 8 == 0 && ((uintptr_t)dy & 15) == 0)
+    k_bias_grad_vec<<<(int)std::max(1ll, std::min<long long>(2 * 152, M / 64)), 256, 0, st>>>(M, C, dy, dys, dyo, db);
+  else
+    k_bias_grad<<<dim3(64, C), 256, 0, st>>>(M, C, dy, dys, dyo, db);
+}
 
 }  // namespace
 }  // namespace dynot
@@ -973,7 +1043,7 @@ ot_status ot_nn_conv3d_wgrad(int N, int T, int Y, int X, int Cin, int Cout, cons
     if (wgrad_tcgen05(N, T, Y, X, Cin, Cout, x, xs, xo, dy, dys, dyo, dw, st, &s2)) {
       if (s2 != OT_OK) return s2;
       if (db) {
-        k_bias_grad<<<dim3(64, Cout), 256, 0, st>>>(M, Cout, (const bf16*)dy, dys, dyo, db);
+        launch_bias_grad(M, Cout, (const bf16*)dy, dys, dyo, db, st);
         NN_LAUNCH_CHECK();
       }
       return OT_OK;
@@ -993,13 +1063,13 @@ ot_status ot_nn_conv3d_wgrad(int N, int T, int Y, int X, int Cin, int Cout, cons
       k_conv3d_wgrad_tiled<<<dim3(nblk, nslices), 128, 0, st>>>(v, Cin, Cout, (const bf16*)x, xs, xo,
                                                                  (const bf16*)dy, dys, dyo, part, (int)ntiles);
       const cudaError_t e1 = cudaGetLastError();
-      if (e1 == cudaSuccess) k_wgrad_reduce<<<dim3(27, nslices), 256, 0, st>>>(Cin, nblk, part, dw);
+      if (e1 == cudaSuccess) k_wgrad_reduce<<<dim3(27 * 256 / 32, nslices), 256, 0, st>>>(Cin, nblk, part, dw);
       const cudaError_t e2 = cudaGetLastError();
       CUDA_OK(cudaFreeAsync(part, st));
       if (e1 != cudaSuccess || e2 != cudaSuccess)
         return seterr(OT_ECUDA, "%s", cudaGetErrorString(e1 != cudaSuccess ? e1 : e2));
       if (db) {
-        k_bias_grad<<<dim3(64, Cout), 256, 0, st>>>(M, Cout, (const bf16*)dy, dys, dyo, db);
+        launch_bias_grad(M, Cout, (const bf16*)dy, dys, dyo, db, st);
         NN_LAUNCH_CHECK();
       }
       return OT_OK;
@@ -1011,7 +1081,7 @@ ot_status ot_nn_conv3d_wgrad(int N, int T, int Y, int X, int Cin, int Cout, cons
       v, Cin, Cout, (const bf16*)x, xs, xo, (const bf16*)dy, dys, dyo, dw, chunk);
   NN_LAUNCH_CHECK();
   if (db) {
-    k_bias_grad<<<dim3(64, Cout), 256, 0, st>>>(M, Cout, (const bf16*)dy, dys, dyo, db);
+    launch_bias_grad(M, Cout, (const bf16*)dy, dys, dyo, db, st);
     NN_LAUNCH_CHECK();
   }
   return OT_OK;
@@ -1025,7 +1095,12 @@ ot_status ot_nn_rotate_weights(int Cin, int Cout, const void* w, void* wr, void*
 }
 
 ot_status ot_nn_relu_grad(long long M, int C, void* g, int gs, int go, const void* y, int ys, int yo, void* stream) {
-  k_relu_grad<<<blocks_for(M * C), 256, 0, (cudaStream_t)stream>>>(M, C, (bf16*)g, gs, go, (const bf16*)y, ys, yo);
+  // 16-byte pieces where the slices allow them; other slices channel by channel
+  if (C % 8 == 0 && gs % 8 == 0 && go % 8 == 0 && ys % 8 == 0 && yo % 8 == 0 && (((uintptr_t)g | (uintptr_t)y) & 15) == 0)
+    k_relu_grad_vec<<<blocks_for(M * (C / 8)), 256, 0, (cudaStream_t)stream>>>(M, C / 8, (bf16*)g, gs, go, (const bf16*)y,
+                                                                             ys, yo);
+  else
+    k_relu_grad<<<blocks_for(M * C), 256, 0, (cudaStream_t)stream>>>(M, C, (bf16*)g, gs, go, (const bf16*)y, ys, yo);
   NN_LAUNCH_CHECK();
   return OT_OK;
 }
