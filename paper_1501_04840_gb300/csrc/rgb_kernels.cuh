@@ -1043,8 +1043,11 @@ __device__ __forceinline__ void update_tiled_body(const Geo<T>& g, const Arrays<
     const bool write_plane = t < tend;
     const bool tnext = t + 1 < g.P;
     T bb[C][4], bn[C][4], xr[C][4], phn[C];
-    // loads of this plane (all channels first, so that they overlap)
-    v4<T> la[C], lb4[C];
+    // loads of this plane (all channels first, so that they overlap; a check's weights too)
+    v4<T> la[C], lb4[C], lw[CHECK ? C : 1];
+    if (CHECK && out && write_plane)
+#pragma unroll
+      for (int c = 0; c < C; ++c) lw[c] = A.w[col + pt + c * sc];
     T phy[C], phd[C], la1d[C], la0l[C], phl[C];
 #pragma unroll
     for (int c = 0; c < C; ++c) {
@@ -1115,7 +1118,7 @@ __device__ __forceinline__ void update_tiled_body(const Geo<T>& g, const Arrays<
         r_db.add(db2);
         r_kx.add(k0 * k0 + k1 * k1 + k2 * k2 + k3 * k3);
         if (V > T(0)) r_J.add(fdiv_fast(U0 * U0 + U1 * U1 + U2 * U2, T(2) * V));
-        const v4<T> wv = A.w[col + pt + c * sc];
+        const v4<T> wv = lw[c];
         r_w.add(bn[c][0] * wv.x + bn[c][1] * wv.y + bn[c][2] * wv.z + bn[c][3] * wv.w);
       }
     }
@@ -1178,7 +1181,7 @@ __device__ __forceinline__ void update_tiled_body(const Geo<T>& g, const Arrays<
 // PXY: the edge blocks handle periodic x / y (a separate instance, so that the Neumann kernel keeps its
 // register allocation)
 template <typename T, int C, bool CHECK, bool WRITE_X, bool PXY>
-__global__ void __launch_bounds__(kTX * kTY, DYNOT_UPD_MINB) k_update_tiled(Geo<T> g, Arrays<T> A, int TC,
+__global__ void __launch_bounds__(kTX * kTY, CHECK ? DYNOT_UPD_MINB - 1 : DYNOT_UPD_MINB) k_update_tiled(Geo<T> g, Arrays<T> A, int TC,
                                                                 TileLayout Lt, double* __restrict__ part) {
   __shared__ T sbb[2][kTY][kTX][C];   // bbar_y exchange, double-buffered by plane parity
   __shared__ double smass[64];

@@ -187,6 +187,11 @@ __device__ __forceinline__ void update_tma_body(const Geo<float>& g, const Array
     const int pt = t * S;
     const bool write_plane = t < tend;
     const bool tnext = t + 1 < g.P;
+    // a check's weights, on their way before the plane's operands are waited for
+    float4 lw[CHECK ? C : 1];
+    if (CHECK && out && write_plane)
+#pragma unroll
+      for (int c = 0; c < C; ++c) lw[c] = A.w[col + pt + c * sc];
     // once a wait has run out, this thread stops waiting (the error is already recorded below)
     if (ok) ok = mbar_wait(bar_ab(slot), (k >> 1) & 1);
     if (ok) ok = mbar_wait(bar_p(ps), (k / 3) & 1);
@@ -259,7 +264,7 @@ __device__ __forceinline__ void update_tma_body(const Geo<float>& g, const Array
         r_db.add(db2);
         r_kx.add(k0 * k0 + k1 * k1 + k2 * k2 + k3 * k3);
         if (V > 0.f) r_J.add(fdiv_fast(U0 * U0 + U1 * U1 + U2 * U2, 2.f * V));
-        const float4 wv = A.w[col + pt + c * sc];
+        const float4 wv = lw[c];
         r_w.add(bn[c][0] * wv.x + bn[c][1] * wv.y + bn[c][2] * wv.z + bn[c][3] * wv.w);
       }
     }
@@ -322,7 +327,7 @@ __device__ __forceinline__ void update_tma_body(const Geo<float>& g, const Array
 }
 
 template <int C, bool CHECK, bool WRITE_X>
-__global__ void __launch_bounds__(kTX * kTY, DYNOT_UPD_MINB)
+__global__ void __launch_bounds__(kTX * kTY, CHECK ? DYNOT_UPD_MINB - 1 : DYNOT_UPD_MINB)
     k_update_tma(Geo<float> g, Arrays<float> A, int TC, double* __restrict__ part, int* __restrict__ err,
                  const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                  const __grid_constant__ CUtensorMap tmP) {
