@@ -459,6 +459,11 @@ struct Plan final : PlanBase {
     const bool split = sx && std::strcmp(sx, "1") == 0;
     mx = mm_shape(n1, g.per1);
     my = mm_shape(n2, g.per2);
+    // The FP64 pipe takes a warp's instruction in the same time whatever its active lanes, and it bounds the FP64 plan:
+    // the products halve the multiply-adds of the dense sums (whose lanes are all busy), so more than half of their
+    // lanes have to be busy too.
+    constexpr bool fp64 = sizeof(T) == 8;
+    auto lanes = [](int items) { return items / (32.0 * ((items + 31) / 32)); };
     const int bufx = mm_buf(mx.l0, mx.lf, mx.li), bufy = mm_buf(my.l0, my.lf, my.li);
     auto round = [](int n, int lo, int hi) { return std::max(lo, std::min(hi, (n + 31) / 32 * 32)); };
     if (!x_fft() && !split) {
@@ -467,7 +472,8 @@ struct Plan final : PlanBase {
       smMx = mm_xt_smem<T>(n1, P, pm, bufx, true);
       smMi = mm_xt_smem<T>(n1, P, pm, bufx, false);
       // (the kernels' offsets into a problem's a are 32-bit)
-      if ((int)smMx <= maxsm && (int)old <= maxsm && 4 * N < (1ll << 31)) {
+      if ((int)smMx <= maxsm && (int)old <= maxsm && 4 * N < (1ll << 31) &&
+          (!fp64 || lanes((P + 7) / 8 * (mx.lf / 4)) > 0.5)) {
         x_mm = true;
         kmf = pick_kmf<T>(pm);
         kmi = pick_kmi<T>(pm);
@@ -482,9 +488,22 @@ struct Plan final : PlanBase {
     }
     if (!y_fft()) {
       const int wt = mm_yc_wt(C);
+      double best = 0.5;
       for (int w = 16; w >= wt; w /= 2) {
         const int items = mm_yc_items(my.lf, C, w);
         const size_t sm = mm_yc_smem<T>(n2, C, w, bufy);
+        if (fp64) {
+          // the share of lanes and columns at work decides (40x48x3x32: strips of 4 columns keep 12 lanes of a warp busy)
+          const double use = lanes(items) * n1 / ((n1 + w - 1) / w * w);
+          if (items > kMmYcThreads || (int)sm > maxsm || use <= best) continue;
+          best = use;
+          y_mm = true;
+          wMy = w;
+          smMy = sm;
+          kmy = pick_kmy<T>(C);
+          ntMy = round(items, 64, kMmYcThreads);
+          continue;
+        }
         // narrower strips while the grid has fewer than three blocks per SM (180x135x3x24: 40.0 us with 8 columns, 42.5
         // with 16; 300x200x3x16: 63.2 against 67.2)
         const bool more = w > wt && (long long)((n1 + w - 1) / w) * P * B < 3 * 152;

@@ -1,6 +1,9 @@
 // Kernels of one PDHG iteration (Algorithm 1) on the grid with three spatial
 // axes x (n1), y (n2), colour (C) and P time intervals.
 //
+// The FP32 plan takes the transform passes of fft_kernels.cuh (FFT lengths) and mm_kernels.cuh (other lengths); K_A to
+// K_C here serve the FP64 plan on FFT lengths and grids that fit neither.
+//
 //   K_A  rhs_fwd_xt : r = A a - f_b^-  (section 3, step 1), then the forward
 //                     DCT-II along x and along t, per (y, c) row of a problem.
 //   K_B  solve_yc   : forward DCT-II along y, the colour eigen-solve with the
@@ -84,7 +87,7 @@ __device__ __forceinline__ double quot_low(double a, double b) {
 // them, good to about 1e-7 of |e| + d + z.  From there Newton converges quadratically from either side (q is
 // increasing and convex for z >= max(e, 0), |q''| / (2 q') <= 2): an FP64 step of size s leaves at most 2 s^2 plus
 // what its approximate reciprocal leaves (1e-6 s), so two steps reach rounding and the loop is for starts that
-// cancellation in e + d spoiled.  Update kernel of the FP64 plan at 128x128x3, P = 32: see k_update_tiled.
+// cancellation in e + d spoiled.  Update kernel of the FP64 plan at 128x128x3, P = 32: 1065 -> 545 us.
 __device__ __forceinline__ double prox_root(double e, double d) {
   const float ef = (float)e, df = (float)d, cf = 1.f + ef;
   const float cbd = cbrt_start(df);
@@ -1179,7 +1182,7 @@ __device__ __forceinline__ void update_tiled_body(const Geo<T>& g, const Arrays<
 }
 
 // PXY: the edge blocks handle periodic x / y (a separate instance, so that the Neumann kernel keeps its
-// register allocation)
+// register allocation).  Checks are compiled for one block per SM less: their sums spilled at 80 registers.
 template <typename T, int C, bool CHECK, bool WRITE_X, bool PXY>
 __global__ void __launch_bounds__(kTX * kTY, CHECK ? DYNOT_UPD_MINB - 1 : DYNOT_UPD_MINB) k_update_tiled(Geo<T> g, Arrays<T> A, int TC,
                                                                 TileLayout Lt, double* __restrict__ part) {
