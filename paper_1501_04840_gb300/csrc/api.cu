@@ -299,17 +299,18 @@ ot_status ot_batch_solve(ot_batch_t b, const float* const* f0, const float* cons
     if (!b || !f0 || !f1 || iters < 1) return seterr(OT_EINVAL, "bad batch solve arguments");
     const int count = (int)b->grp.size();
     for (int i = 0; i < count; ++i) OT_TRY(b->groups[b->grp[i]]->stage_problem(b->idx[i], f0[i], f1[i]));
+    // every problem starts active, before the Poisson solve of the dual weights (in prepare_staged) needs it; one that
+    // meets tol at a check is retired: its kernels return at once from then on, so its state and path stay those of that
+    // check
+    std::vector<std::vector<int>> act(b->groups.size());
+    for (size_t i = 0; i < b->groups.size(); ++i) {
+      act[i].assign(b->groups[i]->B, 1);
+      OT_TRY(b->groups[i]->set_active(act[i], b->groups[i]->st));
+    }
     for (auto& g : b->groups) OT_TRY(g->prepare_staged());   // validation, rescaling, cold start
     for (size_t i = 0; i < b->groups.size(); ++i) {
       CUDA_OK(cudaEventRecord(b->join[i], b->groups[i]->st));
       CUDA_OK(cudaStreamWaitEvent(b->main, b->join[i], 0));
-    }
-    // every problem starts active; one that meets tol at a check is retired: its kernels return at once
-    // from then on, so its state and path stay those of that check
-    std::vector<std::vector<int>> act(b->groups.size());
-    for (size_t i = 0; i < b->groups.size(); ++i) {
-      act[i].assign(b->groups[i]->B, 1);
-      OT_TRY(b->groups[i]->set_active(act[i], b->main));
     }
     std::vector<int> its(count, 0);
     int live = count;
