@@ -128,8 +128,9 @@ __global__ void k_unpack_path(Geo<T> g, Compact cp, const float* __restrict__ pa
 template <typename T>
 __device__ __forceinline__ float scaled(T v, double scale, float sh, float sl) {
   if constexpr (sizeof(T) == 4) {
-    if (sh == 0.f) return (float)((double)v * scale);
     const float p = v * sh;
+    // the FP64 product where the parts of the scale do not fit, and for infinities (p - p would make NaN of them)
+    if (sh == 0.f || !isfinite(p)) return (float)((double)v * scale);
     return p + fmaf(v, sl, fmaf(v, sh, -p));
   } else {
     return (float)((double)v * scale);
