@@ -156,9 +156,17 @@ struct KSum {
   }
 };
 
+// FP64 sum over the lanes of a warp, in every lane
+__device__ __forceinline__ double warp_sum64(double d) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+  return d;
+}
+
 // A sum carried in two values of the working precision: every addition keeps its rounding error (Knuth's two-sum) and
-// every product its own (a fused multiply-add), so FP32 terms and sums are good to about 2^-45.  The FP64 pipe is a
-// sixty-fourth of the FP32 one: five FP64 additions per warp and plane took longer than the rest of a residual check.
+// every product its own (a fused multiply-add), so FP32 terms and sums are good to about 2^-45 while they stay inside the
+// FP32 range (fitting_total below takes FP64 where they do not).  The FP64 pipe is a sixty-fourth of the FP32 one: five
+// FP64 additions per warp and plane took longer than the rest of a residual check.
 template <typename T>
 struct Sum2 {
   T hi = T(0), lo = T(0);
@@ -172,7 +180,13 @@ struct Sum2 {
     lo += fma(a, b, -p);
     add(p);
   }
-  // the sum over the lanes of a warp, in every lane
+  // (a - b)^2 of the exact difference, good to 2^-45 as well
+  __device__ __forceinline__ void add_square_of_difference(T a, T b) {
+    const T s = a - b, v = s - a, e = (a - (s - v)) - (b + v);
+    add_product(s, s);
+    lo = fma(T(2) * s, e, lo);
+  }
+  // the sum over the lanes of a warp; in FP64 where lanes that are finite sum to more than T holds
   __device__ __forceinline__ double warp_total() const {
     Sum2 t = *this;
 #pragma unroll
@@ -181,8 +195,21 @@ struct Sum2 {
       t.add(h);
       t.lo += l;
     }
+    if (__any_sync(0xffffffffu, !isfinite(t.hi))) return warp_sum64((double)hi + (double)lo);
     return (double)t.hi + (double)t.lo;
   }
 };
+
+// Warp total of a sum of products whose magnitudes add up to `size` in this lane: the two-value sum where no product and
+// no remainder that matters has left the FP32 range (a remainder lost to underflow is below 2^-149, a lane at 1e30 cannot
+// overflow the warp), the sum of exact() (this lane's terms in FP64) otherwise.  Called by whole warps.
+template <typename T, class F>
+__device__ __forceinline__ double fitting_total(const Sum2<T>& s, T size, F&& exact) {
+  if constexpr (sizeof(T) == 4) {
+    const bool some = __any_sync(0xffffffffu, size > 1e-20f), all = __all_sync(0xffffffffu, size < 1e30f);
+    if (!(some && all)) return warp_sum64(exact());
+  }
+  return s.warp_total();
+}
 
 }  // namespace dynot

@@ -322,10 +322,10 @@ __global__ void __launch_bounds__(128) k_update(Geo<T> g, Arrays<T> A, double* _
   if (retired(g, b)) return;
   pdl_wait();   // phi and the state are read from here on
   const bool live = x < g.n1;
-  Sum2<T> r_db, r_kx, r_J, r_m, r_w;
+  T bn[4] = {}, kx[4] = {}, bo[4] = {}, wk[4] = {}, U0 = T(0), U1 = T(0), U2 = T(0), V = T(0), f = T(0);
   if (live) {
     CellCtx<T> cc{g, A, b};
-    T bb[4], bn[4], xrr[4], kx[4], U0, U1, U2, V;
+    T bb[4], xrr[4];
     cc.cell(t, x, y, c, bb, bn, xrr, kx, U0, U1, U2, V);
     const size_t i0 = cidx(g, b, t, x, y, c);
     T an[4];
@@ -358,33 +358,64 @@ __global__ void __launch_bounds__(128) k_update(Geo<T> g, Arrays<T> A, double* _
     A.bn[i0] = mk4<T>(bn[0], bn[1], bn[2], bn[3]);
     if (WRITE_X) A.x[i0] = mk4<T>(xrr[0], xrr[1], xrr[2], xrr[3]);
     if (CHECK) {
-      const v4<T> bo4 = A.b[i0];
-      const T bo[4] = {bo4.x, bo4.y, bo4.z, bo4.w};
-      const v4<T> wv = A.w[i0];
-      const T wk[4] = {wv.x, wv.y, wv.z, wv.w};
+      const v4<T> bo4 = A.b[i0], wv = A.w[i0];
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        const T db = bn[k] - bo[k];
-        r_db.add_product(db, db);
-        r_kx.add_product(kx[k], kx[k]);
-        r_w.add_product(bn[k], wk[k]);
+        bo[k] = cget<T>(bo4, k);
+        wk[k] = cget<T>(wv, k);
       }
-      if (V > T(0)) {
-        // |u|^2 / (2 v), the quotient with its remainder
-        Sum2<T> uu;
-        uu.add_product(U0, U0);
-        uu.add_product(U1, U1);
-        uu.add_product(U2, U2);
-        const T v2 = T(2) * V, q = uu.hi / v2;
-        r_J.hi = q;
-        r_J.lo = (fma(-q, v2, uu.hi) + uu.lo) / v2;
-      }
-      r_m.add(xrr[3]);
+      f = xrr[3];
     }
   }
   if (CHECK) {
     __shared__ double red[4][5];
-    const double d[5] = {r_db.warp_total(), r_kx.warp_total(), r_J.warp_total(), r_m.warp_total(), r_w.warp_total()};
+    Sum2<T> r_db, r_kx, r_J, r_m, r_w, uu;
+    T size_w = T(0);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      r_db.add_square_of_difference(bn[k], bo[k]);
+      r_kx.add_product(kx[k], kx[k]);
+      r_w.add_product(bn[k], wk[k]);
+      size_w += fabs(bn[k] * wk[k]);
+    }
+    uu.add_product(U0, U0);
+    uu.add_product(U1, U1);
+    uu.add_product(U2, U2);
+    T size_J = T(0);
+    if (V > T(0)) {
+      // |u|^2 / (2 v), the quotient with its remainder (FP64 for a v that could raise what underflow took from |u|^2)
+      const T v2 = T(2) * V, q = uu.hi / v2;
+      r_J.hi = q;
+      r_J.lo = (fma(-q, v2, uu.hi) + uu.lo) / v2;
+      size_J = V < T(1e-18) ? T(INFINITY) : q;
+    }
+    r_m.add(f);
+    const double d[5] = {
+        fitting_total<T>(r_db, r_db.hi, [&] {
+          double s = 0;
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const double db = (double)bn[k] - (double)bo[k];
+            s += db * db;
+          }
+          return s;
+        }),
+        fitting_total<T>(r_kx, r_kx.hi, [&] {
+          double s = 0;
+#pragma unroll
+          for (int k = 0; k < 4; ++k) s += (double)kx[k] * (double)kx[k];
+          return s;
+        }),
+        fitting_total<T>(r_J, size_J, [&] {
+          return V > T(0) ? ((double)U0 * U0 + (double)U1 * U1 + (double)U2 * U2) / (2.0 * (double)V) : 0.0;
+        }),
+        r_m.warp_total(),
+        fitting_total<T>(r_w, size_w, [&] {
+          double s = 0;
+#pragma unroll
+          for (int k = 0; k < 4; ++k) s += (double)bn[k] * (double)wk[k];
+          return s;
+        })};
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
     if (l == 0)
 #pragma unroll
@@ -940,8 +971,8 @@ struct TileLayout {
 };
 
 // Per-block partial sums of a check (called by every thread of a 32 x 8 block after its plane loop):
-// sums of the threads' compensated partials (two-value sums in a warp, FP64 across warps), written to
-// part[problem][quantity][block].
+// sums of the threads' compensated partials (two-value sums in a warp, FP64 where they would overflow and across warps),
+// written to part[problem][quantity][block].
 template <typename T>
 __device__ __forceinline__ void block_check_partials(const KSum<T>& r_db, const KSum<T>& r_kx, const KSum<T>& r_J,
                                                      const KSum<T>& r_w, int lane, int row, int nch, int b, int t0,
