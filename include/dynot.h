@@ -362,12 +362,12 @@ ot_status ot_nn_dual_channels(int N, int Y, int X, int P, int to_channels, float
  *   renormalised to mass 1; integer counts by largest remainders).  The paper cites its circular specification method without
  *   printing it; the reading implemented: pixels ranked by (hue, index), rank
  *   r gets target rank (r - s) mod npix, where the cyclic shift s has the least
- *   squared circular distance of all npix shifts (ties to the
- *   smaller shift; for sorted points on the circle an optimal matching under a
+ *   squared circular distance of all npix shifts (the smaller of shifts whose
+ *   computed costs are equal; for sorted points on the circle an optimal matching under a
  *   cost convex in the distance is such a shift), and target rank q in bin b
  *   gets the hue (b + (q - C_b + 1/2) / c_b) / bins.  Allocates its workspace
- *   and synchronises `stream`; 1 <= npix <= 2^21 (hues in [0, 1] are
- *   searched in about 1400 npix terms, others in npix^2).
+ *   and synchronises `stream`; 1 <= npix <= 2^21 (images of more than
+ *   2048 pixels and more than one hue, all in [0, 1], are searched in about 1400 npix terms, others in npix^2).
  */
 ot_status ot_rgb_to_hsv(int npix, const float* rgb, float* h, float* s, float* v, void* stream);
 ot_status ot_hsv_to_rgb(int npix, const float* h, const float* s, const float* v, float* rgb, void* stream);

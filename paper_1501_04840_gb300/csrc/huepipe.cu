@@ -9,7 +9,7 @@
 // remainders, ties to the lower bin); target rank q in bin b gets the hue
 // (b + (q - C_b + 1/2) / c_b) / bins; the circle is cut at the cyclic shift s of
 // least squared circular distance sum_r d(x_r, y_{(r-s) mod n})^2 over all n
-// shifts (ties to the smaller shift).  For sorted points on the circle and a
+// shifts (the smaller of shifts whose computed costs are equal).  For sorted points on the circle and a
 // cost convex in the circular distance an optimal matching is a cyclic shift of
 // the sorted orders, so this cut is the optimal assignment of the source pixels
 // to the target hues.
@@ -193,9 +193,11 @@ __global__ void k_target_hues(int n, int bins, const long long* __restrict__ C, 
 //   k_shift_window  : the costs of the kShiftBlock shifts around it, tile by tile in float;
 //   k_window_costs  : their sums over the tiles in double, in order; k_argmin_shift takes the least.
 // The costs are the sums of the exhaustive search below term by term, so the shift is the one it finds (rounding
-// moves a minimum of the float sums by a few shifts, the window holds 512 to either side).  n^2 terms become about
-// 1400 n: 0.08 ms in place of 4.7 ms for 65536 pixels.  Hues outside [0, 1] (k_shift_inputs finds them) and images
-// of at most kShiftSmall pixels take the exhaustive search, which covers every shift.
+// moves a minimum of the float sums by a few shifts, the window holds 512 to either side; costs that agree to float
+// rounding over more shifts than that are told apart by their rounding alone).  n^2 terms become about 1400 n: 0.08 ms
+// in place of 4.7 ms for 65536 pixels.  Hues outside [0, 1], images of one hue (all shifts cost the
+// same there, and the first minimum of the float sums may lie anywhere) and images of at most kShiftSmall pixels take
+// the exhaustive search, which covers every shift.
 //
 // Exhaustive search and window alike: a block takes
 // kShiftBlock consecutive shifts, kShiftPer per thread (s = s0 + tid + kShiftThreads u), and walks r in
@@ -389,11 +391,11 @@ __global__ void k_argmin_shift(int n, const double* __restrict__ cost, const int
 }
 
 // float source hues of the sorted ranks, the target hues as float pairs and their gaps; sets *all where a hue lies
-// outside [0, 1] or the image is small, so that every shift is searched
+// outside [0, 1], or the image is small or of one hue, so that every shift is searched
 __global__ void k_shift_inputs(int n, const double* __restrict__ x, const double* __restrict__ y,
                                float* __restrict__ xs, float2* __restrict__ ys, float* __restrict__ gap,
                                int* __restrict__ all) {
-  if (n <= kShiftSmall && blockIdx.x == 0 && threadIdx.x == 0) *all = 1;
+  if ((n <= kShiftSmall || x[0] == x[n - 1]) && blockIdx.x == 0 && threadIdx.x == 0) *all = 1;
   for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
     xs[r] = (float)x[r];
     const float hi = (float)y[r];
@@ -537,7 +539,7 @@ ot_status ot_hue_specify(int npix, const float* h, int bins, const float* target
     CUDA_OK(cudaMemcpyAsync(dC, C.data(), sizeof(long long) * (bins + 1), cudaMemcpyHostToDevice, st));
     k_target_hues<<<grid_for(npix), 256, 0, st>>>(npix, bins, dC, y);
     HP_CHECK();
-    // least-cost cyclic shift over all npix shifts
+    // least-cost cyclic shift: by convexity, or over all npix shifts
     k_shift_inputs<<<grid_for(npix), 256, 0, st>>>(npix, x, y, xs, ys, dgap, dall);
     HP_CHECK();
     for (int k = 0; k < kSlopeRounds; ++k) k_shift_slope<<<kSlopePoints, 256, 0, st>>>(npix, k, xs, dgap, y, dneg);
