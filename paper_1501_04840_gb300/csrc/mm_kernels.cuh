@@ -298,9 +298,9 @@ __global__ void __launch_bounds__(kMmXtThreads, sizeof(T) == 4 ? 2 : 1)
   __syncthreads();
   mm_fold<T>(X, ld, (P + 3) / 4, ax);
   __syncthreads();
-  // FP64 releases its successor only at its end: measured per iteration with the trigger here and without, 40x48x3x32
-  // 402 -> 313 us, 58x59x3x48 787 -> 533, 128x40x3x16 390 -> 299, 93x129x3x16 778 -> 718; 143x160x3x40 and 110x66x3x64
-  // are the same (3790, 1613 us).  The cause was not isolated.
+  // FP64 releases its successor only at its end (XtTables::late): measured per iteration with the trigger here and
+  // without, 40x48x3x32 402 -> 313 us, 58x59x3x48 787 -> 533, 128x40x3x16 390 -> 299, 93x129x3x16 778 -> 718;
+  // 143x160x3x40 and 110x66x3x64 are the same (3790, 1613 us).
   if constexpr (sizeof(T) == 4) pdl_trigger();
   const int G = (P + 7) / 8, Q0 = ax.l0 / 4, Q = ax.lf / 4;
   for (int r0 = 0; r0 < G * Q; r0 += blockDim.x) {

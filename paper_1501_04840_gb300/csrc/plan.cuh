@@ -449,9 +449,19 @@ struct Plan final : PlanBase {
     return OT_OK;
   }
 
+  // Multiply-adds of the FP64 pipe on the busiest quarter of an SM, in warp instructions: `blocks` blocks of `warps`
+  // warps, `steps` instructions each.  The pipe takes a warp's instruction in the same time whatever its active lanes.
+  static long long fp64_load(long long blocks, long long warps, long long steps) {
+    constexpr int sms = 152, quarters = 4;
+    return ((blocks + sms - 1) / sms * warps + quarters - 1) / quarters * steps;
+  }
+  static long long warps_of(long long items) { return (items + 31) / 32; }
+
   // Axes without an FFT length take the folded products where a (x, t) plane (x) or a strip of columns (y) fits
-  // shared memory and a strip's outputs fit one block's registers; the dense sums keep the rest (axes beyond about
-  // 1500 cells, and planes that the dense passes hold but this layout does not).
+  // shared memory and a strip's outputs fit one block's registers; the dense sums keep the rest.  In FP32 that is x axes
+  // beyond 1093 cells (P = 9), 760 (P = 24), 624 (P = 32), 458 (P = 48) or 359 (P = 64) and y axes beyond 1024; in FP64
+  // half of that or less.  The FP64 plan also keeps the dense sums where they load the pipe less: the products halve the
+  // multiply-adds, but a thread holds 32 to 48 sums, and short axes leave most of an SM's quarters without a warp.
   ot_status choose_mm() {
     int maxsm = 0;
     CUDA_OK(cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, device));
@@ -459,43 +469,53 @@ struct Plan final : PlanBase {
     const bool split = sx && std::strcmp(sx, "1") == 0;
     mx = mm_shape(n1, g.per1);
     my = mm_shape(n2, g.per2);
-    // The FP64 pipe takes a warp's instruction in the same time whatever its active lanes, and it bounds the FP64 plan:
-    // the products halve the multiply-adds of the dense sums (whose lanes are all busy), so more than half of their
-    // lanes have to be busy too.
     constexpr bool fp64 = sizeof(T) == 8;
     auto lanes = [](int items) { return items / (32.0 * ((items + 31) / 32)); };
     const int bufx = mm_buf(mx.l0, mx.lf, mx.li), bufy = mm_buf(my.l0, my.lf, my.li);
     auto round = [](int n, int lo, int hi) { return std::max(lo, std::min(hi, (n + 31) / 32 * 32)); };
     if (!x_fft() && !split) {
-      const int pm = mm_pm(P), dense = 4 * n1;
+      const int pm = mm_pm(P), dense = 4 * n1, G = (P + 7) / 8;
       const size_t old = xt_layout<T>(nullptr, nullptr, P, n1, pmax, dense, true);
       smMx = mm_xt_smem<T>(n1, P, pm, bufx, true);
       smMi = mm_xt_smem<T>(n1, P, pm, bufx, false);
+      // Both passes, the time transforms included.  Measured (us, forward and inverse pass, dense | products): 63, P = 9
+      // 52 | 97; 33x2x3, P = 12 46 | 64; 150x24x3, P = 12 182 | 212; 40x48x3, P = 32 146 | 114; 110x66x3, P = 64 1430 |
+      // 785.  400 instructions (13 us) are what the products' barriers and table copies cost beside them.
+      const long long nb = (long long)n2 * C * B, cols = warps_of(n1), P4 = (P + 3) / 4 * 4, hP4 = ((P + 1) / 2 + 3) / 4 * 4;
+      const bool less = fp64_load(nb, cols, P4 * pm / 2 + hP4 * pm) + fp64_load(nb, warps_of(G * (mx.lf / 4)), 32ll * mx.h0) +
+                            fp64_load(nb, warps_of(G * ((mx.h0 + 1) / 2)), 32ll * mx.h0) + 400 <
+                        fp64_load(nb, cols, 2ll * P * pmax) + fp64_load(nb, 8 * ((P * n1 + 255) / 256), 2ll * n1);
       // (the kernels' offsets into a problem's a are 32-bit)
-      if ((int)smMx <= maxsm && (int)old <= maxsm && 4 * N < (1ll << 31) &&
-          (!fp64 || lanes((P + 7) / 8 * (mx.lf / 4)) > 0.5)) {
+      if ((int)smMx <= maxsm && (int)old <= maxsm && 4 * N < (1ll << 31) && (!fp64 || less)) {
         x_mm = true;
         kmf = pick_kmf<T>(pm);
         kmi = pick_kmi<T>(pm);
-        // threads: the columns of the time transform or the products' items, whichever are more
-        const int G = (P + 7) / 8;
         // threads: the products' items in equal rounds, up to 160 (three or four blocks per SM) where the grid fills the
         // GPU and as many as have work otherwise
-        const int most = (long long)n2 * C * B > 2 * 152 ? 160 : kMmXtThreads;
+        const int most = nb > 2 * 152 ? 160 : kMmXtThreads;
         const int work = G * (mx.lf / 4), rounds = (work + most - 1) / most;
         ntMf = ntMi = round(std::max((work + rounds - 1) / rounds, std::min(n1, 96)), 64, most);
       }
     }
     if (!y_fft()) {
       const int wt = mm_yc_wt(C);
-      double best = 0.5;
+      // FP64: the load of the dense sums (strips of kW columns, both transforms) less what the products' folding, barriers
+      // and copies cost beside them, about 200 instructions and a twentieth.  Measured (us, dense | products):
+      // 32x30x3, P = 9 27 | 75; 128x40x3, P = 16 65 | 96; 40x48x3, P = 32 80 | 100; 64x150x1, P = 16 111 | 193;
+      // 128x75x3, P = 24 253 | 225; 58x59x3, P = 48 166 | 146; 143x160x3, P = 40 1637 | 1181; 36x160x3, P = 25 342 | 399
+      // with strips of 16 columns, 305 with 8.  Between strips of the same load the share of lanes and columns at work
+      // decides (100x100x1, P = 32 141 us with 16 columns, 133 with 8).
+      double load = fp64_load((long long)((n1 + kW - 1) / kW) * P * B, 8 * ((kW * C * n2 + 255) / 256), 2ll * n2) / 0.95 - 200;
+      double best = 0;
       for (int w = 16; w >= wt; w /= 2) {
         const int items = mm_yc_items(my.lf, C, w);
         const size_t sm = mm_yc_smem<T>(n2, C, w, bufy);
         if (fp64) {
-          // the share of lanes and columns at work decides (40x48x3x32: strips of 4 columns keep 12 lanes of a warp busy)
+          const long long nb = (long long)((n1 + w - 1) / w) * P * B, steps = 4ll * wt * C * my.h0;
+          const double l = (double)(fp64_load(nb, warps_of(items), steps) + fp64_load(nb, warps_of(w / wt * ((my.h0 + 1) / 2)), steps));
           const double use = lanes(items) * n1 / ((n1 + w - 1) / w * w);
-          if (items > kMmYcThreads || (int)sm > maxsm || use <= best) continue;
+          if (items > kMmYcThreads || (int)sm > maxsm || l > load || (l == load && use <= best)) continue;
+          load = l;
           best = use;
           y_mm = true;
           wMy = w;
@@ -775,6 +795,7 @@ struct Plan final : PlanBase {
         ax.it = (const T*)(base + off[1]);
       };
       if (x_mm) mm_ptrs(mx, o_mx);
+      xt.late = sizeof(T) == 8 && !(x_fft() && y_fft());
       mtf = (const T*)(base + o_mtf);
       mti = (const T*)(base + o_mti);
       if (y_mm) mm_ptrs(my, o_my);

@@ -457,6 +457,12 @@ struct XtTables {
   const void* cos4;  // [4 n1]; for a periodic x axis the (cos, sin)(2 pi m / n1) pairs instead
   const void* twt;   // c2<T>[P]: exp(-2 pi i j / P)   (register t-DCT when P == PMAX <= 32)
   const void* hwt;   // c2<T>[P]: exp(-i pi k / (2P))
+  // FP64 grids with an axis that has no FFT: the passes on either side of its products and dense sums release their
+  // successor at their end.  Released early, the next pass's blocks settle on whichever SMs are free, several to one,
+  // while a few FP64-bound blocks want an SM each: 64x150x1, P = 16 616 us an iteration whose passes add up to 316, 295
+  // like this; 96x130x1, P = 20 616 -> 337; 64x40x3, P = 16 with dense sums along y 269 -> 149.  Both axes by FFT keep
+  // the early release (256x256x3, P = 32 3478 us against 3483 without any).
+  int late;
 };
 
 // The time transform runs in registers by FFT when P fills the template width
@@ -592,7 +598,7 @@ __global__ void __launch_bounds__(256, DYNOT_XT_MINB) k_rhs_fwd_xt(Geo<T> g, con
     dct_cols<T, PMAX>(s.tile, n1, n1, P, s.Mt);
   }
   __syncthreads();
-  pdl_trigger();
+  if (sizeof(T) == 4 || (N1 > 0 && !tb.late)) pdl_trigger();
   store_tile_rows<T>(s.tile, rhat + cidx(g, b, 0, 0, y, c), (size_t)g.S, P, n1);
 }
 
@@ -761,7 +767,7 @@ __global__ void __launch_bounds__(256, DYNOT_XTC_MINB) k_inv_xt(Geo<T> g, const 
     if (g.per1) rdft_dense_rows<T, false>(rows, P, n1, true, (T*)s.scr, 2 * scr_elems, (const c2<T>*)s.cos4);
     else dct_dense_rows<T, false>(rows, P, n1, true, (T*)s.scr, 2 * scr_elems, s.cos4);
   }
-  pdl_trigger();
+  if constexpr (sizeof(T) == 4 || N1 > 0) pdl_trigger();   // (FP64: see XtTables::late)
   store_tile_rows<T>(s.tile, phi + cidx(g, b, 0, 0, y, c), (size_t)g.S, P, n1);
 }
 
@@ -923,7 +929,7 @@ __global__ void __launch_bounds__(NT, 768 / NT) k_solve_yc(Geo<T> g, T* __restri
     if (g.per2) rdft_dense_rows<T, true>(rows, nrows, n2, true, (T*)scr, 2 * scr_elems, (const c2<T>*)cos4);
     else dct_dense_rows<T, true>(rows, nrows, n2, true, (T*)scr, 2 * scr_elems, cos4);
   }
-  pdl_trigger();
+  if constexpr (sizeof(T) == 4 || M1 > 0) pdl_trigger();   // (FP64: see XtTables::late)
   for (int c = 0; c < C; ++c) {
     T* dst = hat + plane + (size_t)c * n1 * n2;
     const T* src = tile + c * cst;
