@@ -199,8 +199,8 @@ __global__ void __launch_bounds__(256) k_hue_inv(Geo<T> g, const T* __restrict__
 //   k_hue_x_inv : the inverse real DFT -> phi, 8 rows x 2 mirrored pairs per thread.
 // SMALL (few rows, a single pair) is bound by latency: blocks of 8 rows x 64 outputs whose table columns are copied
 // while the previous kernel runs, every sum in 16 slices of at most n / 32 steps.  Otherwise the FP32 pipe and the
-// instructions around it bound: 16 rows x all outputs per block, tables in chunks of 8 steps, sums in runs of 16 terms
-// (which keep the rounding error of 16 + n / 32 additions).
+// instructions around it bound: 16 or 8 rows x all outputs or some per block, tables in chunks of K = 8 or 16 steps, sums
+// in runs of 16 terms (which keep the rounding error of 16 + n / 32 additions).  plan.cuh (choose_hue_mm) picks.
 // ---------------------------------------------------------------------------
 constexpr int kHueMmThreads = 256;
 constexpr int kHueSlices = 16, kHueItems = 16;   // SMALL: slices of a sum, items (64 table columns) per block
@@ -208,16 +208,16 @@ constexpr int kHueSlices = 16, kHueItems = 16;   // SMALL: slices of a sum, item
 // Rows of X before and after the bins, so that whole steps of 16 stay inside: their table weights are zero.
 __host__ __device__ inline int hue_hpad(int h0) { return (h0 + 15) / 16 * 16; }
 __host__ __device__ inline int hue_xpad(int n, int h0) { return hue_hpad(h0) > n ? hue_hpad(h0) - n : 0; }
-inline size_t hue_mm_vals(int n, int h0, int rb, int items, bool small) {
+inline size_t hue_mm_vals(int n, int h0, int rb, int items, bool small, int K = kMmK) {
   const size_t x = (size_t)(n + 2 * hue_xpad(n, h0)) * (rb + 4);
   const size_t tab = (size_t)hue_hpad(h0) * 4 * kHueItems, red = (size_t)kHueSlices * 32 * kHueItems;
-  return x + (small ? (tab > red ? tab : red) : (size_t)kMmStages * kMmK * 4 * items);
+  return x + (small ? (tab > red ? tab : red) : (size_t)kMmStages * K * 4 * items);
 }
 
-// Copies of `width` columns of a table (row stride ld) in chunks of 8 rows into slots of row stride ldb.  The place of a
+// Copies of `width` columns of a table (row stride ld) in chunks of K rows into slots of row stride ldb.  The place of a
 // thread's first vector and the step between its vectors are found once (a division per vector and chunk took a
 // quarter of the kernel's instructions).
-template <typename T>
+template <typename T, int K>
 struct HueChunks {
   const T* tab;
   T* buf;
@@ -231,10 +231,10 @@ struct HueChunks {
     dk = blockDim.x - dr * per;
   }
   __device__ __forceinline__ void issue(int c) const {
-    if (c * kMmK >= hpad) return;
-    T* dst = buf + (c % kMmStages) * kMmK * ldb;
-    const T* src = tab + (size_t)c * kMmK * ld;
-    for (int i = r, j = k; i < kMmK;) {
+    if (c * K >= hpad) return;
+    T* dst = buf + (c % kMmStages) * K * ldb;
+    const T* src = tab + (size_t)c * K * ld;
+    for (int i = r, j = k; i < K;) {
       cp_async16(dst + i * ldb + V * j, src + i * ld + V * j);
       i += dr;
       j += dk;
@@ -285,7 +285,7 @@ __device__ __forceinline__ void hue_cells(int rows, int n, F&& f) {
   }
 }
 
-template <typename T, bool SMALL>
+template <typename T, bool SMALL, int K>
 __global__ void __launch_bounds__(kHueMmThreads, sizeof(T) == 4 ? 2 : 1)
     k_hue_x_fwd(Geo<T> g, const v4<T>* __restrict__ ap, const T* __restrict__ f0, const T* __restrict__ f1,
                 T* __restrict__ hat, MmAxis<T> ax, int RB, int QC) {
@@ -297,7 +297,7 @@ __global__ void __launch_bounds__(kHueMmThreads, sizeof(T) == 4 ? 2 : 1)
   T* X = (T*)smraw + pad * ld;
   T* buf = X + (n + pad) * ld;
   const T* tab = ax.ft + 4 * u0;
-  const HueChunks<T> chunks(buf, tab, ax.lf, 4 * qn, 4 * QC, hpad);
+  const HueChunks<T, K> chunks(buf, tab, ax.lf, 4 * qn, 4 * QC, hpad);
   if (SMALL) {
     hue_columns<T>(buf, tab, ax.lf, qn, 4 * kHueItems, hpad);
   } else {
@@ -385,15 +385,15 @@ __global__ void __launch_bounds__(kHueMmThreads, sizeof(T) == 4 ? 2 : 1)
   mm_zero<T>(acc);
   mm_zero<T>(part);
 #pragma unroll 1
-  for (int c = 0; c * kMmK < hpad; ++c) {
+  for (int c = 0; c * K < hpad; ++c) {
     asm volatile("cp.async.wait_group 1;\n" ::: "memory");
     __syncthreads();   // chunk c is there (and, at first, the folded rows), and every thread is done with chunk c - 1
     chunks.issue(c + 2);
     hue_commit();
     if (!live) continue;
-    const T* tc = buf + (c % kMmStages) * kMmK * 4 * QC + 4 * u;
+    const T* tc = buf + (c % kMmStages) * K * 4 * QC + 4 * u;
 #pragma unroll
-    for (int j = 0; j < kMmK; ++j) {
+    for (int j = 0; j < K; ++j) {
       T v[8], m[4];
       ldv<T, 8>(row, v);
       ldv<T, 4>(tc, m);
@@ -404,7 +404,7 @@ __global__ void __launch_bounds__(kHueMmThreads, sizeof(T) == 4 ? 2 : 1)
 #pragma unroll
         for (int e = 0; e < 4; ++e) part[r][e] = fma(v[r], m[e], part[r][e]);
     }
-    if (c & 1) {
+    if (K == 16 || (c & 1)) {   // 16 terms
 #pragma unroll
       for (int r = 0; r < 8; ++r)
 #pragma unroll
@@ -427,7 +427,7 @@ __global__ void __launch_bounds__(kHueMmThreads, sizeof(T) == 4 ? 2 : 1)
     }
 }
 
-template <typename T, bool SMALL>
+template <typename T, bool SMALL, int K>
 __global__ void __launch_bounds__(kHueMmThreads, sizeof(T) == 4 ? 2 : 1)
     k_hue_x_inv(Geo<T> g, const T* __restrict__ hat, T* __restrict__ phi, MmAxis<T> ax, int RB, int IC) {
   extern __shared__ __align__(16) char smraw[];
@@ -437,8 +437,8 @@ __global__ void __launch_bounds__(kHueMmThreads, sizeof(T) == 4 ? 2 : 1)
   const int hpad = hue_hpad(ax.h0), pad = hue_xpad(n, ax.h0);
   T* X = (T*)smraw + pad * ld;   // [slot][t]
   T* buf = X + (n + pad) * ld;
-  const HueChunks<T> ce(buf, ax.it + i00, 2 * ax.li, wid, 4 * IC, hpad);
-  const HueChunks<T> co(buf + 2 * IC, ax.it + ax.li + i00, 2 * ax.li, wid, 4 * IC, hpad);
+  const HueChunks<T, K> ce(buf, ax.it + i00, 2 * ax.li, wid, 4 * IC, hpad);
+  const HueChunks<T, K> co(buf + 2 * IC, ax.it + ax.li + i00, 2 * ax.li, wid, 4 * IC, hpad);
   auto issue = [&](int c) {
     ce.issue(c);
     co.issue(c);
@@ -520,15 +520,15 @@ __global__ void __launch_bounds__(kHueMmThreads, sizeof(T) == 4 ? 2 : 1)
   mm_zero<T>(acc);
   mm_zero<T>(part);
 #pragma unroll 1
-  for (int c = 0; c * kMmK < hpad; ++c) {
+  for (int c = 0; c * K < hpad; ++c) {
     asm volatile("cp.async.wait_group 1;\n" ::: "memory");
     __syncthreads();
     issue(c + 2);
     if (!live) continue;
-    const T* tc = buf + (c % kMmStages) * kMmK * 4 * IC + 2 * u;
+    const T* tc = buf + (c % kMmStages) * K * 4 * IC + 2 * u;
 #pragma unroll
-    for (int j = 0; j < kMmK; ++j) {
-      const int q = c * kMmK + j;
+    for (int j = 0; j < K; ++j) {
+      const int q = c * K + j;
       T v[8], m[2];
       ldv<T, 8>(even + q * ld, v);
       ldv<T, 2>(tc, m);
@@ -544,7 +544,7 @@ __global__ void __launch_bounds__(kHueMmThreads, sizeof(T) == 4 ? 2 : 1)
         for (int e = 0; e < 2; ++e) part[r][2 + e] = fma(v[r], m[e], part[r][2 + e]);
       tc += 4 * IC;
     }
-    if (c & 1) {
+    if (K == 16 || (c & 1)) {   // 16 terms
 #pragma unroll
       for (int r = 0; r < 8; ++r)
 #pragma unroll

@@ -140,7 +140,7 @@ struct Plan final : PlanBase {
   int ntMf = 0, ntMi = 0, ntMy = 0, wMy = 0;
   // hue transforms as folded products (hue_kernels.cuh); mx holds the bins' tables
   struct HueLaunch {
-    int rb = 8, chunk = 0, nch = 1, nt = 0;
+    int rb = 8, chunk = 0, nch = 1, nt = 0, k = kMmK;   // rows and items per block, blocks per row group, steps per chunk
     size_t smem = 0;
   };
   bool hue_mm = false, hue_small = false;
@@ -417,38 +417,6 @@ struct Plan final : PlanBase {
     return ax;
   }
 
-  // The hue transforms as folded products, where the rows fit shared memory (3000 bins do).  Fewer row groups than
-  // SMs (a single pair): the latency-bound form of the kernels, where its table columns fit.
-  ot_status choose_hue_mm() {
-    int maxsm = 0;
-    CUDA_OK(cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, device));
-    mx = mm_shape(n1, true);
-    const int items_f = mx.lf / 4, items_i = (mx.h0 + 1) / 2;   // outputs per 8 rows, 4 table columns each
-    auto pick = [&](int items, int even) {
-      HueLaunch h;
-      h.rb = !hue_small && P > 8 ? 16 : 8;
-      if (hue_small) {
-        h.chunk = kHueItems;
-        h.nt = kHueMmThreads;
-      } else {
-        const int cap = kHueMmThreads / (h.rb / 8), nch = (items + cap - 1) / cap;
-        h.chunk = ((items + nch - 1) / nch + even - 1) / even * even;
-        h.nt = std::max(128, (h.rb / 8 * h.chunk + 31) / 32 * 32);
-      }
-      h.nch = (items + h.chunk - 1) / h.chunk;
-      h.smem = sizeof(T) * hue_mm_vals(n1, mx.h0, h.rb, h.chunk, hue_small);
-      return h;
-    };
-    const long long G8 = (long long)((P + 7) / 8) * B;
-    hue_small = G8 < 152 && (int)(sizeof(T) * hue_mm_vals(n1, mx.h0, 8, kHueItems, true)) <= maxsm;
-    hf = pick(items_f, 1);
-    hi = pick(items_i, 2);
-    hsc = hue_small ? HueTt<true>::SC : HueTt<false>::SC;
-    smTt = sizeof(T) * hue_tt_vals(P, hsc);
-    hue_mm = (int)std::max(std::max(hf.smem, hi.smem), smTt) <= maxsm && hf.nt <= kHueMmThreads && hi.nt <= kHueMmThreads;
-    return OT_OK;
-  }
-
   // Multiply-adds of the FP64 pipe on the busiest quarter of an SM, in warp instructions: `blocks` blocks of `warps`
   // warps, `steps` instructions each.  The pipe takes a warp's instruction in the same time whatever its active lanes.
   static long long fp64_load(long long blocks, long long warps, long long steps) {
@@ -456,6 +424,89 @@ struct Plan final : PlanBase {
     return ((blocks + sms - 1) / sms * warps + quarters - 1) / quarters * steps;
   }
   static long long warps_of(long long items) { return (items + 31) / 32; }
+
+  // The hue transforms as folded products, where the rows fit shared memory (at 16 rows per block and P > 8 up to 2339
+  // bins in FP32; not every length below the last that fits: the chunks of an axis differ).
+  //  - Few row groups (a single pair): the latency-bound form of the kernels, where its table columns fit and, in FP32,
+  //    its blocks, which form their 8 rows' r again for every 16 items, run in at most four waves (720 bins, P = 32:
+  //    8 pairs in 3 waves 61 us an iteration against 71, 16 pairs in 6 waves 101 against 82).
+  //  - FP32: 16 rows per block and the fewest chunks of items, the least table traffic, where these blocks fill the GPU;
+  //    as many chunks as two blocks per SM hold where they would leave some SMs with two blocks and some with one
+  //    (850 bins, P = 40, 32 pairs 196 -> 174 us).  Fewer blocks: 8 rows, and chunks (of a warp's lanes at least) up to
+  //    one block per SM (720 bins, 16 pairs 101 -> 82 us; 1000 bins, P = 64, 8 pairs 140 -> 120).
+  //  - FP32: steps in chunks of 16, which wait half as often for copies, unless fewer blocks would share an SM
+  //    (1000 bins, P = 64, 64 pairs 640 -> 593 us; 500 bins, 64 pairs would take 192 instead of 173).
+  //  - FP64: the per-row kernels where they load the FP64 pipe less (720 bins, P = 32, one pair 1331 -> 326 us;
+  //    180 bins, P = 36, 32 pairs 366 -> 345; 360 bins, P = 64, one pair keeps the products, 95 against 133).
+  ot_status choose_hue_mm() {
+    int maxsm = 0, smsm = 0, reserved = 0;
+    CUDA_OK(cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, device));
+    CUDA_OK(cudaDeviceGetAttribute(&smsm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, device));
+    CUDA_OK(cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, device));
+    constexpr bool fp64 = sizeof(T) == 8;
+    constexpr int sms = 152;
+    mx = mm_shape(n1, true);
+    const int items_f = mx.lf / 4, items_i = (mx.h0 + 1) / 2;   // outputs per 8 rows, 4 table columns each
+    const long long G8 = (long long)((P + 7) / 8) * B, G16 = (long long)((P + 15) / 16) * B;
+    const size_t smem_small = sizeof(T) * hue_mm_vals(n1, mx.h0, 8, kHueItems, true);
+    auto resident = [&](size_t smem, int nt) {   // blocks per SM, at 128 registers
+      return std::max<long long>(1, std::min<long long>(smsm / ((long long)smem + reserved), 65536 / (128 * nt)));
+    };
+    auto waves = [&](int items) {
+      const long long per = sms * resident(smem_small, kHueMmThreads);
+      return (G8 * ((items + kHueItems - 1) / kHueItems) + per - 1) / per;
+    };
+    hue_small = G8 < sms && (int)smem_small <= maxsm && (fp64 || std::max(waves(items_f), waves(items_i)) <= 4);
+    auto pick = [&](int items, int even) {
+      HueLaunch h;
+      if (hue_small) {
+        h.chunk = kHueItems;
+        h.nt = kHueMmThreads;
+        h.nch = (items + h.chunk - 1) / h.chunk;
+        h.smem = smem_small;
+        return h;
+      }
+      auto least = [&](int rb) { return (items + kHueMmThreads / (rb / 8) - 1) / (kHueMmThreads / (rb / 8)); };
+      h.rb = P > 8 ? 16 : 8;
+      h.nch = least(h.rb);
+      if (!fp64) {
+        if (P > 8 && G16 * h.nch < 92) h.rb = 8;
+        if (h.rb == 8) {
+          h.nch = std::max<int>(least(8), (int)std::min<long long>(sms / G8, items / 32));
+        } else if (G16 * h.nch > sms) {
+          h.nch = std::max<int>(h.nch, (int)(2 * sms / G16));
+        }
+      }
+      h.chunk = ((items + h.nch - 1) / h.nch + even - 1) / even * even;
+      h.nch = (items + h.chunk - 1) / h.chunk;
+      h.nt = std::max(128, (h.rb / 8 * h.chunk + 31) / 32 * 32);
+      h.smem = sizeof(T) * hue_mm_vals(n1, mx.h0, h.rb, h.chunk, false);
+      if (!fp64) {
+        const size_t s16 = sizeof(T) * hue_mm_vals(n1, mx.h0, h.rb, h.chunk, false, 16);
+        const long long per_sm = ((h.rb == 8 ? G8 : G16) * h.nch + sms - 1) / sms;
+        if ((int)s16 <= maxsm && resident(s16, h.nt) >= std::min(per_sm, resident(h.smem, h.nt))) {
+          h.k = 16;
+          h.smem = s16;
+        }
+      }
+      return h;
+    };
+    hf = pick(items_f, 1);
+    hi = pick(items_i, 2);
+    hsc = hue_small ? HueTt<true>::SC : HueTt<false>::SC;
+    smTt = sizeof(T) * hue_tt_vals(P, hsc);
+    hue_mm = (int)std::max(std::max(hf.smem, hi.smem), smTt) <= maxsm && hf.nt <= kHueMmThreads && hi.nt <= kHueMmThreads;
+    if (fp64 && hue_mm) {
+      // both bin transforms and the time transforms (P^2 or, per row, 2 P pmax multiply-adds per slot)
+      const long long hpad = hue_hpad(mx.h0), cols = (long long)n1 * B * P / (32 * 4 * sms);
+      auto load = [&](const HueLaunch& h) {
+        return hue_small ? fp64_load(G8 * h.nch, kHueMmThreads / 32, 32 * hpad / kHueSlices)
+                         : fp64_load((long long)((P + h.rb - 1) / h.rb) * B * h.nch, warps_of(h.rb / 8 * h.chunk), 32 * hpad);
+      };
+      hue_mm = load(hf) + load(hi) + cols * P <= 1.05 * (fp64_load((long long)P * B, warps_of(n1), 2ll * n1) + cols * 2 * pmax);
+    }
+    return OT_OK;
+  }
 
   // Axes without an FFT length take the folded products where a (x, t) plane (x) or a strip of columns (y) fits
   // shared memory and a strip's outputs fit one block's registers; the dense sums keep the rest.  In FP32 that is x axes
@@ -870,8 +921,12 @@ struct Plan final : PlanBase {
         mx.ft = (const T*)(base + o_mx[0]);
         mx.it = (const T*)(base + o_mx[1]);
         htt = (const T*)(base + o_tt);
-        for (const void* f : {(const void*)k_hue_x_fwd<T, true>, (const void*)k_hue_x_fwd<T, false>, (const void*)k_hue_x_inv<T, true>,
-                              (const void*)k_hue_x_inv<T, false>, (const void*)k_hue_tt<T, true>, (const void*)k_hue_tt<T, false>})
+        if constexpr (sizeof(T) == 4)
+          for (const void* f : {(const void*)k_hue_x_fwd<T, false, 16>, (const void*)k_hue_x_inv<T, false, 16>})
+            CUDA_OK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, maxsm));
+        for (const void* f : {(const void*)k_hue_x_fwd<T, true, kMmK>, (const void*)k_hue_x_fwd<T, false, kMmK>,
+                              (const void*)k_hue_x_inv<T, true, kMmK>, (const void*)k_hue_x_inv<T, false, kMmK>,
+                              (const void*)k_hue_tt<T, true>, (const void*)k_hue_tt<T, false>})
           CUDA_OK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, maxsm));
       }
     }
@@ -945,13 +1000,19 @@ struct Plan final : PlanBase {
     } else {
       if (evs) cudaEventRecord(evs[0], st);
       if (hue_mm) {
-        launch_pdl(hue_small ? k_hue_x_fwd<T, true> : k_hue_x_fwd<T, false>, dim3((P + hf.rb - 1) / hf.rb, hf.nch, B),
+        auto xf = hue_small ? k_hue_x_fwd<T, true, kMmK> : k_hue_x_fwd<T, false, kMmK>;
+        auto xi = hue_small ? k_hue_x_inv<T, true, kMmK> : k_hue_x_inv<T, false, kMmK>;
+        if constexpr (sizeof(T) == 4) {
+          if (hf.k == 16) xf = k_hue_x_fwd<T, false, 16>;
+          if (hi.k == 16) xi = k_hue_x_inv<T, false, 16>;
+        }
+        launch_pdl(xf, dim3((P + hf.rb - 1) / hf.rb, hf.nch, B),
                    dim3(hf.nt), hf.smem, st, g, asrc, (const T*)f0n, (const T*)f1n, hat, mx, hf.rb, hf.chunk);
         if (evs) cudaEventRecord(evs[1], st);
         launch_pdl(hue_small ? k_hue_tt<T, true> : k_hue_tt<T, false>, dim3((n1 + hsc - 1) / hsc, B), dim3(256), smTt, st,
                    g, hat, ht, htt);
         if (evs) cudaEventRecord(evs[2], st);
-        launch_pdl(hue_small ? k_hue_x_inv<T, true> : k_hue_x_inv<T, false>, dim3((P + hi.rb - 1) / hi.rb, hi.nch, B),
+        launch_pdl(xi, dim3((P + hi.rb - 1) / hi.rb, hi.nch, B),
                    dim3(hi.nt), hi.smem, st, g, (const T*)hat, phi, mx, hi.rb, hi.chunk);
       } else {
         k_hue_fwd<T><<<dim3(P, B), 256, smH, st>>>(g, asrc, f0n, f1n, hat, ht);
