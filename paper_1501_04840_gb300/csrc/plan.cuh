@@ -645,54 +645,26 @@ struct Plan final : PlanBase {
       }
       return l;
     };
-    auto mm_axis = [&](const MmAxis<T>& ax, size_t (&off)[2]) {
+    // Its tables, zero up to whole groups of 16 rows (read by the hue kernels), are filled on the device (k_mm_tables) behind
+    // the host's; off: turn, turn2, then ft and it from the end of the host's tables.
+    size_t dev = 0;
+    auto mm_axis = [&](const MmAxis<T>& ax, size_t (&off)[4]) {
       const int n = ax.n;
-      const bool per = ax.o1;
-      // cos(2 pi m / (4 n)) over a full turn (sin: m + 3 n); along a table row the index m advances by a constant
       std::vector<T> turn(4 * n), turn2(4 * n);
       for (int m = 0; m < 4 * n; ++m) {
         const double v = std::cos(2 * kPi * m / (4.0 * n));
         turn[m] = (T)v;
         turn2[m] = (T)(2.0 / n * v);
       }
-      auto fill = [&](T* dst, int cnt, const std::vector<T>& tab, long long m0, long long step) {
-        int m = (int)(m0 % (4 * n)), d = (int)(step % (4 * n));
-        for (int i = 0; i < cnt; ++i) {
-          dst[i] = tab[m];
-          m += d;
-          if (m >= 4 * n) m -= 4 * n;
-        }
-      };
-      const size_t rows = hue_hpad(ax.h0);   // zero rows up to whole groups of 16 (read by the hue kernels)
-      std::vector<T> tf(rows * ax.lf, T(0)), ti(rows * 2 * ax.li, T(0));
-      for (int i = 0; i < ax.h0; ++i) {
-        T* row = tf.data() + (size_t)i * ax.lf;
-        if (per) {   // cos(2 pi q i / n); sin(2 pi (q + 1) (i + 1) / n)
-          fill(row, ax.h0, turn, 0, 4ll * i);
-          if (i < ax.h1) fill(row + ax.l0, ax.h1, turn, 4ll * (i + 1) + 3ll * n, 4ll * (i + 1));
-        } else {     // cos(pi k (2 i + 1) / (2 n)) for k = 2 q and 2 q + 1
-          fill(row, ax.h0, turn, 0, 2ll * (2 * i + 1));
-          if (i < ax.h1) fill(row + ax.l0, ax.h1, turn, 2 * i + 1, 2ll * (2 * i + 1));
-        }
-      }
-      for (int q = 0; q < ax.h0; ++q) {
-        T* row = ti.data() + (size_t)q * 2 * ax.li;
-        const int k = mm_freq(n, per, q);
-        const bool one = k == 0 || (per && 2 * k == n);   // weight 1 / n, all others 2 / n
-        if (per) {
-          fill(row, ax.h0, turn2, 0, 4ll * q);
-          if (q < ax.h1) fill(row + ax.li, ax.h0, turn2, 3ll * n, 4ll * (q + 1));
-        } else {
-          fill(row, ax.h0, turn2, k, 2ll * k);
-          if (q < ax.h1) fill(row + ax.li, ax.h0, turn2, k + 1, 2ll * (k + 1));
-        }
-        if (one)
-          for (int i = 0; i < ax.h0; ++i) row[i] *= T(0.5);
-      }
-      off[0] = put(tf.data(), tf.size() * sizeof(T));
-      off[1] = put(ti.data(), ti.size() * sizeof(T));
+      off[0] = put(turn.data(), turn.size() * sizeof(T));
+      off[1] = put(turn2.data(), turn2.size() * sizeof(T));
+      const size_t rows = hue_hpad(ax.h0);
+      off[2] = dev;
+      dev += rnd16(rows * ax.lf * sizeof(T));
+      off[3] = dev;
+      dev += rnd16(rows * 2 * ax.li * sizeof(T));
     };
-    size_t o_mx[2] = {}, o_my[2] = {}, o_mtf = 0, o_mti = 0;
+    size_t o_mx[4] = {}, o_my[4] = {}, o_mtf = 0, o_mti = 0;
     // (cos, sin)(2 pi m / n) pairs, padded to the 4 n values of the cosine table they replace
     auto cs_pad = [&](int n) {
       std::vector<T> c(4 * n, T(0));
@@ -707,6 +679,9 @@ struct Plan final : PlanBase {
       for (size_t i = 0; i < v.size(); ++i) r[i] = (T)v[i];
       return r;
     };
+    // cos(pi m / 2P), for the folded time transforms
+    std::vector<double> cosP(4 * P);
+    for (int m = 0; m < 4 * P; ++m) cosP[m] = std::cos(kPi * (double)m / (2.0 * P));
     // time axis: forward and inverse DCT matrices, padded to pmax columns
     std::vector<T> Mf((size_t)P * pmax, T(0)), Mi((size_t)P * pmax, T(0));
     for (int k = 0; k < P; ++k)
@@ -754,7 +729,7 @@ struct Plan final : PlanBase {
         std::vector<T> tf((size_t)P4 * ph, T(0)), ti((size_t)hP4 * pm, T(0));
         for (int k = 0; k < P; ++k)
           for (int t = 0; t < P; ++t) {
-            const double c = std::cos(kPi * (double)(k * (2 * t + 1) % (4 * P)) / (2.0 * P));
+            const double c = cosP[k * (2 * t + 1) % (4 * P)];
             if (t < hP) tf[(size_t)k * ph + t] = (T)c;
             if (t < hP4) ti[(size_t)t * pm + (k & 1) * ph + k / 2] = (T)((k == 0 ? 1.0 : 2.0) / P * c);
           }
@@ -811,7 +786,7 @@ struct Plan final : PlanBase {
         T *te = tt.data() + (size_t)hP * P4, *to = te + (size_t)hP * h4;
         for (int k = 0; k < P; ++k)
           for (int t = 0; t < hP; ++t) {
-            const double c = std::cos(kPi * (double)(k * (2 * t + 1) % (4 * P)) / (2.0 * P));
+            const double c = cosP[k * (2 * t + 1) % (4 * P)];
             tt[(size_t)t * P4 + k] = (T)c;
             (k & 1 ? to : te)[(size_t)(k / 2) * h4 + t] = (T)((k == 0 ? 1.0 : 2.0) / P * c);
           }
@@ -828,9 +803,18 @@ struct Plan final : PlanBase {
       o_hl = put(hlT.data(), n * sizeof(T));
       o_hld = put(hl.data(), n * sizeof(double));
     }
-    CUDA_OK(cudaMalloc(&tabmem.p, h.size()));
-    CUDA_OK(cudaMemcpy(tabmem.p, h.data(), h.size(), cudaMemcpyHostToDevice));
+    CUDA_OK(cudaMalloc(&tabmem.p, h.size() + dev));
+    CUDA_OK(cudaMemcpyAsync(tabmem.p, h.data(), h.size(), cudaMemcpyHostToDevice, st));
     char* base = (char*)tabmem.p;
+    auto mm_fill = [&](MmAxis<T>& ax, const size_t (&off)[4]) -> ot_status {
+      T *ft = (T*)(base + h.size() + off[2]), *it = (T*)(base + h.size() + off[3]);
+      ax.ft = ft;
+      ax.it = it;
+      k_mm_tables<T><<<dim3((ax.lf + 2 * ax.li + 127) / 128, hue_hpad(ax.h0)), 128, 0, st>>>(
+          ax, (const T*)(base + off[0]), (const T*)(base + off[1]), ft, it);
+      CUDA_OK(cudaGetLastError());
+      return OT_OK;
+    };
     if (!hue) {
       xt.tw = base + o_tw1; xt.hw = base + o_hw1; xt.cos4 = base + o_c41;
       xt.Mt_f = base + o_Mf; xt.Mt_i = base + o_Mi;
@@ -841,15 +825,11 @@ struct Plan final : PlanBase {
       yc.lamtd = (const double*)(base + o_ltd);
       yc.Qc = base + o_Q; yc.lamc = base + o_lc; yc.lamcd = (const double*)(base + o_lcd);
       yc.lam_fp64 = thr;
-      auto mm_ptrs = [&](MmAxis<T>& ax, const size_t (&off)[2]) {
-        ax.ft = (const T*)(base + off[0]);
-        ax.it = (const T*)(base + off[1]);
-      };
-      if (x_mm) mm_ptrs(mx, o_mx);
+      if (x_mm) OT_TRY(mm_fill(mx, o_mx));
       xt.late = sizeof(T) == 8 && !(x_fft() && y_fft());
       mtf = (const T*)(base + o_mtf);
       mti = (const T*)(base + o_mti);
-      if (y_mm) mm_ptrs(my, o_my);
+      if (y_mm) OT_TRY(mm_fill(my, o_my));
       scrA = x_fft() ? (kThreadsXt / fft_n1(n1)) * n1 : 4 * n1;
       scrB = y_fft() ? (yc_threads(n2) / fft_n1(n2)) * n2 : 4 * n2;
       ka = pick_ka<T>(x_fft() ? n1 : 0, pmax);
@@ -918,8 +898,7 @@ struct Plan final : PlanBase {
       CUDA_OK(cudaFuncSetAttribute((const void*)k_hue_inv<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxsm));
       CUDA_OK(cudaFuncSetAttribute((const void*)kh, cudaFuncAttributeMaxDynamicSharedMemorySize, maxsm));
       if (hue_mm) {
-        mx.ft = (const T*)(base + o_mx[0]);
-        mx.it = (const T*)(base + o_mx[1]);
+        OT_TRY(mm_fill(mx, o_mx));
         htt = (const T*)(base + o_tt);
         if constexpr (sizeof(T) == 4)
           for (const void* f : {(const void*)k_hue_x_fwd<T, false, 16>, (const void*)k_hue_x_inv<T, false, 16>})
