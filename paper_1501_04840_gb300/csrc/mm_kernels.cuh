@@ -21,7 +21,8 @@
 // iteration 117 against 575 us.  What bounds them there is latency at three blocks per SM (issue slots 36-47 % busy,
 // 1.7 M cells leave 10 warps per SM with this register tile); the multiply-adds alone would take 5-8 us each.
 // They replace the dense sums of k_rhs_fwd_xt, k_solve_yc and k_inv_xt (one output and n dependent steps per
-// thread), which remain for planes that do not fit shared memory in this layout.
+// thread), which remain for planes that do not fit shared memory in this layout and for FP64 grids whose pipe they load
+// less (plan.cuh, choose_mm).
 #pragma once
 #include "rgb_kernels.cuh"
 

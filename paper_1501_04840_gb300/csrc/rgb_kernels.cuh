@@ -58,16 +58,6 @@ __device__ __forceinline__ float cbrt_start(float d) {
 }
 __device__ __forceinline__ double cbrt_start(double d) { return cbrt(d); }
 
-// Per-cell proximal map of J (section 3, step 2):
-//   argmin_{u,v} |u|^2/(2v) + sigma/2 |u - a_m|^2 + sigma/2 (v - a_f)^2.
-// With z = sigma v, e = sigma a_f and d = sigma^2 |a_m|^2 / 2 the cubic of the
-// paper, 2 (1 + sigma v)^2 (v - a_f) = sigma |a_m|^2, reads
-//   q(z) = (1 + z)^2 (z - e) - d = 0,   u = z a_m / (1 + z),  v = z / sigma.
-// A root z > 0 exists iff e + d > 0; otherwise (u, v) = (0, 0).  With w = 1 + z
-// and c = 1 + e the root satisfies w^2 (w - c) = d, which gives the upper
-// bounds w <= c + min(d^(1/3), d/c^2) for c > 0 and w <= min(d^(1/3), sqrt(d/|c|))
-// for c <= 0.  q is increasing and convex for z >= max(e, 0), so Newton's
-// method from that bound decreases monotonically to the root.
 __device__ __forceinline__ double rcp_approx(double x) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
@@ -85,7 +75,7 @@ __device__ __forceinline__ double quot_low(double a, double b) {
   return fma(fma(-b, q, a), r, q);
 }
 
-// The root of q(z) = (1 + z)^2 (z - e) - d in FP64 (e + d > 0; |e| and d far from overflow).  The FP64 pipe is a
+// The root of q(z) = (1 + z)^2 (z - e) - d of the proximal map below in FP64 (e + d > 0; |e| and d far from overflow).  The FP64 pipe is a
 // sixty-fourth of the FP32 one, so the start comes from FP32: bound and three Newton steps as prox_J<float> takes
 // them, good to about 1e-7 of |e| + d + z.  From there Newton converges quadratically from either side (q is
 // increasing and convex for z >= max(e, 0), |q''| / (2 q') <= 2): an FP64 step of size s leaves at most 2 s^2 plus
@@ -117,6 +107,16 @@ __device__ __forceinline__ double prox_root(double e, double d) {
   return z;
 }
 
+// Per-cell proximal map of J (section 3, step 2):
+//   argmin_{u,v} |u|^2/(2v) + sigma/2 |u - a_m|^2 + sigma/2 (v - a_f)^2.
+// With z = sigma v, e = sigma a_f and d = sigma^2 |a_m|^2 / 2 the cubic of the
+// paper, 2 (1 + sigma v)^2 (v - a_f) = sigma |a_m|^2, reads
+//   q(z) = (1 + z)^2 (z - e) - d = 0,   u = z a_m / (1 + z),  v = z / sigma.
+// A root z > 0 exists iff e + d > 0; otherwise (u, v) = (0, 0).  With w = 1 + z
+// and c = 1 + e the root satisfies w^2 (w - c) = d, which gives the upper
+// bounds w <= c + min(d^(1/3), d/c^2) for c > 0 and w <= min(d^(1/3), sqrt(d/|c|))
+// for c <= 0.  q is increasing and convex for z >= max(e, 0), so Newton's
+// method from that bound decreases monotonically to the root.
 template <typename T>
 __device__ __forceinline__ void prox_J(T am0, T am1, T am2, T af, T sigma, T inv_sigma, T& u0, T& u1, T& u2, T& v) {
   const T s2 = am0 * am0 + am1 * am1 + am2 * am2;
