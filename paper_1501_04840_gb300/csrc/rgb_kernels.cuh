@@ -64,15 +64,13 @@ __device__ __forceinline__ double rcp_approx(double x) {
   return r;
 }
 
-// a / b for the low modes, in FP64 to its last place: the approximate reciprocal with one Newton step, the quotient and
-// one step on its remainder.  The blocks that hold the low modes are the last to finish, and a division takes them longer:
-// 64x64x3, P = 32 29.0 us an iteration against 33.8, 128x128x3, P = 32 55.6 against 61.0 (28.5 and 55.2 without the last
-// step, which leaves 2^-40).
+// a / b for the low modes, in FP64 to its last place: with the approximate reciprocal r and its error e = 1 - b r (2^-20),
+// a r (1 + e + e^2), three dependent steps.  The blocks that hold the low modes are the last to finish, and a division
+// takes them longer: 64x64x3, P = 32 28.7 us an iteration against 33.8, 128x128x3, P = 32 55.3 against 61.0 (28.5 and 55.2
+// without e^2, which leaves 2^-40).
 __device__ __forceinline__ double quot_low(double a, double b) {
-  double r = rcp_approx(b);
-  r = fma(fma(-b, r, 1.0), r, r);
-  const double q = a * r;
-  return fma(fma(-b, q, a), r, q);
+  const double r = rcp_approx(b), q = a * r, e = fma(-b, r, 1.0);
+  return fma(q, fma(e, e, e), q);
 }
 
 // The root of q(z) = (1 + z)^2 (z - e) - d of the proximal map below in FP64 (e + d > 0; |e| and d far from overflow).  The FP64 pipe is a
