@@ -18,7 +18,7 @@
 //   k_mm_yc     : the y transform, the colour eigen-solve and divide, the inverse y transform;
 //   k_mm_inv_xt : the inverse time DCT of every column, the inverse x transform -> phi.
 // At 180x135x3, P = 24 (events, one GB300): 36, 40 and 27 us against 138, 185 and 234 us of the dense sums; the
-// iteration 117 against 575 us.  What bounds them there is latency at three blocks per SM (issue slots 36-47 % busy,
+// iteration 117 against 575 us.  What bounds them there is latency at three blocks per SM (issue slots 39-56 % busy,
 // 1.7 M cells leave 10 warps per SM with this register tile); the multiply-adds alone would take 5-8 us each.
 // They replace the dense sums of k_rhs_fwd_xt, k_solve_yc and k_inv_xt (one output and n dependent steps per
 // thread), which remain for planes that do not fit shared memory in this layout and for FP64 grids whose pipe they load

@@ -73,10 +73,10 @@ __device__ __forceinline__ double quot_low(double a, double b) {
   return fma(q, fma(e, e, e), q);
 }
 
-// The root of q(z) = (1 + z)^2 (z - e) - d of the proximal map below in FP64 (e + d > 0; |e| and d far from overflow).  The FP64 pipe is a
-// sixty-fourth of the FP32 one, so the start comes from FP32: bound and three Newton steps as prox_J<float> takes
-// them, good to about 1e-7 of |e| + d + z.  From there Newton converges quadratically from either side (q is
-// increasing and convex for z >= max(e, 0), |q''| / (2 q') <= 2): an FP64 step of size s leaves at most 2 s^2 plus
+// The root of q(z) = (1 + z)^2 (z - e) - d of the proximal map below in FP64 (e + d > 0; |e| and d far from overflow).
+// The FP64 pipe is a sixty-fourth of the FP32 one, so the start comes from FP32: bound and three Newton steps as
+// prox_J<float> takes them, good to about 1e-7 of |e| + d + z.  From there Newton converges quadratically from either side
+// (q is increasing and convex for z >= max(e, 0), |q''| / (2 q') <= 2): an FP64 step of size s leaves at most 2 s^2 plus
 // what its approximate reciprocal leaves (1e-6 s), so two steps reach rounding and the loop is for starts that
 // cancellation in e + d spoiled.  Update kernel of the FP64 plan at 128x128x3, P = 32: 1065 -> 545 us.
 __device__ __forceinline__ double prox_root(double e, double d) {
