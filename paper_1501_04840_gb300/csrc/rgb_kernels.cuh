@@ -392,7 +392,7 @@ __global__ void __launch_bounds__(128) k_update(Geo<T> g, Arrays<T> A, double* _
     }
     r_m.add(f);
     const double d[5] = {
-        fitting_total<T>(r_db, r_db.hi, [&] {
+        fitting_total<T>(r_db, r_db.hi, live, [&] {
           double s = 0;
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
@@ -401,17 +401,17 @@ __global__ void __launch_bounds__(128) k_update(Geo<T> g, Arrays<T> A, double* _
           }
           return s;
         }),
-        fitting_total<T>(r_kx, r_kx.hi, [&] {
+        fitting_total<T>(r_kx, r_kx.hi, live, [&] {
           double s = 0;
 #pragma unroll
           for (int k = 0; k < 4; ++k) s += (double)kx[k] * (double)kx[k];
           return s;
         }),
-        fitting_total<T>(r_J, size_J, [&] {
+        fitting_total<T>(r_J, size_J, V > T(0), [&] {
           return V > T(0) ? ((double)U0 * U0 + (double)U1 * U1 + (double)U2 * U2) / (2.0 * (double)V) : 0.0;
         }),
         r_m.warp_total(),
-        fitting_total<T>(r_w, size_w, [&] {
+        fitting_total<T>(r_w, size_w, live, [&] {
           double s = 0;
 #pragma unroll
           for (int k = 0; k < 4; ++k) s += (double)bn[k] * (double)wk[k];
