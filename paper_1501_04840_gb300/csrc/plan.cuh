@@ -593,9 +593,12 @@ struct Plan final : PlanBase {
   // ---- transform tables (computed in double on the host)
   ot_status build_tables() {
     std::vector<char> h;
+    // tables start on whole lines: a warp's copy of 512 bytes is then four of them (333 bins, P = 27, 32 pairs: the time
+    // transforms 16.6 us from a table that starts between them, 11.8 like this)
+    auto line = [](size_t nb) { return (nb + 255) / 256 * 256; };
     auto put = [&](const void* src, size_t nb) {
       size_t off = h.size();
-      h.resize(off + rnd16(nb));
+      h.resize(off + line(nb));
       std::memcpy(h.data() + off, src, nb);
       return off;
     };
@@ -660,9 +663,9 @@ struct Plan final : PlanBase {
       off[1] = put(turn2.data(), turn2.size() * sizeof(T));
       const size_t rows = hue_hpad(ax.h0);
       off[2] = dev;
-      dev += rnd16(rows * ax.lf * sizeof(T));
+      dev += line(rows * ax.lf * sizeof(T));
       off[3] = dev;
-      dev += rnd16(rows * 2 * ax.li * sizeof(T));
+      dev += line(rows * 2 * ax.li * sizeof(T));
     };
     size_t o_mx[4] = {}, o_my[4] = {}, o_mtf = 0, o_mti = 0;
     // (cos, sin)(2 pi m / n) pairs, padded to the 4 n values of the cosine table they replace
