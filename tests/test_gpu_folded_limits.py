@@ -21,7 +21,7 @@ F64 = [((64, 150, 1), (N, N, N), 16), ((96, 130, 1), (N, N, N), 20), ((63,), (N,
 # bins, P, pairs, precision: few rows in slices, 8 and 16 rows per block, one and several chunks of items, chunks of 8 and
 # 16 steps, per-row kernels
 HUES = [(2339, 9, 1, 0), (2341, 9, 1, 0), (2905, 8, 1, 0), (720, 32, 8, 0), (720, 32, 16, 0), (1000, 64, 8, 0), (1000, 64, 16, 0),
-        (850, 40, 32, 0), (500, 64, 64, 0), (360, 64, 24, 0), (101, 20, 60, 0), (37, 5, 160, 0), (1500, 17, 1, 0),
+        (850, 40, 32, 0), (500, 64, 64, 0), (360, 64, 24, 0), (101, 20, 60, 0), (37, 5, 160, 0), (1500, 17, 1, 0), (4096, 64, 1, 0), (3500, 20, 2, 0),
         (720, 32, 1, 2), (720, 32, 32, 2), (180, 36, 32, 2), (64, 16, 32, 2), (333, 27, 4, 2), (1024, 9, 1, 2)]
 
 
