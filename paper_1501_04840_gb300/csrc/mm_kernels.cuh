@@ -116,7 +116,10 @@ __device__ __forceinline__ void mm_zero(T (&acc)[RT][E]) {
     for (int e = 0; e < E; ++e) acc[r][e] = T(0);
 }
 
-// Tables on their way through shared memory: chunks of kMmK rows in kMmStages slots.
+// Tables on their way through shared memory: chunks of kMmK rows in kMmStages slots.  The slots come first in a block's
+// shared memory, so that they start on lines of 128 bytes as the tables do in global memory: a warp's copy of 512 bytes
+// falls apart into more pieces otherwise (224x97x1, P = 16: y pass 15.8 us, 20.0 with the tables 16 bytes further, 21.7 with
+// the slots 48 bytes off; 180x135x3, P = 24 38.9, 42.5, 42.3).
 constexpr int kMmK = 8, kMmStages = 3;
 __host__ __device__ inline int mm_buf(int l0, int lf, int li) { return kMmStages * kMmK * (lf > 2 * li ? lf : 2 * li); }
 
@@ -241,10 +244,10 @@ __global__ void __launch_bounds__(kMmXtThreads, sizeof(T) == 4 ? 2 : 1)
   const int c = blockIdx.x, y = blockIdx.y, b = blockIdx.z;
   if (retired(g, b)) return;
   const int n1 = g.n1, P = g.P, ld = mm_ldt(P), P4 = (P + 3) / 4 * 4, hP = (P + 1) / 2;
-  T* X = (T*)smraw;          // [x][t]
+  T* buf = (T*)smraw;        // table chunks
+  T* X = buf + mm_buf(ax.l0, ax.lf, ax.li);   // [x][t]
   T* Mt = X + n1 * ld;       // [k][PH]
-  T* buf = Mt + P4 * PH;     // table chunks
-  T* R = buf + mm_buf(ax.l0, ax.lf, ax.li);   // [t][x]
+  T* R = Mt + P4 * PH;       // [t][x]
   mm_start<T>(buf, ax.ft, ax.lf, ax.h0);
   for (int j = threadIdx.x; j < P4 * PH; j += blockDim.x) Mt[j] = Mtg[j];
   __syncthreads();
@@ -371,9 +374,9 @@ __global__ void __launch_bounds__(kMmXtThreads, sizeof(T) == 4 ? 2 : 1)
   const int y = blockIdx.x, c = blockIdx.y, b = blockIdx.z;
   if (retired(g, b)) return;
   const int n1 = g.n1, P = g.P, ld = mm_ldt(P), hP = (P + 1) / 2, hP4 = (hP + 3) / 4 * 4;
-  T* X = (T*)smraw;          // [spectral x][t]
+  T* buf = (T*)smraw;        // table chunks
+  T* X = buf + mm_buf(ax.l0, ax.lf, ax.li);   // [spectral x][t]
   T* Mt = X + n1 * ld;
-  T* buf = Mt + (P + 3) / 4 * 4 * PM;   // table chunks
   mm_start<T>(buf, ax.it, 2 * ax.li, ax.h0);
   for (int j = threadIdx.x; j < hP4 * PM; j += blockDim.x) Mt[j] = Mtg[j];
   __syncthreads();
@@ -474,8 +477,8 @@ __global__ void __launch_bounds__(kMmYcThreads, sizeof(T) == 4 ? 2 : 1) k_mm_yc(
   if (retired(g, b)) return;
   const int n1 = g.n1, n2 = g.n2, ld = (C * W + 7) / 8 * 8 + 4, NW = W / WT;
   const int w_act = min(W, n1 - x0);
-  T* X = (T*)smraw;          // [y][wg][c][wi]
-  T* buf = X + n2 * ld;      // table chunks
+  T* buf = (T*)smraw;        // table chunks
+  T* X = buf + mm_buf(ay.l0, ay.lf, ay.li);   // [y][wg][c][wi]
   mm_start<T>(buf, ay.ft, ay.lf, ay.h0);
   T Q[C][C], lc[C];
 #pragma unroll
@@ -486,7 +489,7 @@ __global__ void __launch_bounds__(kMmYcThreads, sizeof(T) == 4 ? 2 : 1) k_mm_yc(
   }
   const T lt = ((const T*)tb.lamt)[kt];
   const double ltd = tb.lamtd[kt];
-  T* l2 = buf + mm_buf(ay.l0, ay.lf, ay.li);   // eigenvalues along y and x (the strip), also in double
+  T* l2 = X + n2 * ld;       // eigenvalues along y and x (the strip), also in double
   T* l1 = l2 + n2;
   double* l2d = (double*)(((uintptr_t)(l1 + W) + 7) & ~uintptr_t(7));
   double* l1d = l2d + n2;
