@@ -17,8 +17,8 @@
 //   k_mm_fwd_xt : r = A a - f_b^-, the time DCT of every column in registers, the x transform;
 //   k_mm_yc     : the y transform, the colour eigen-solve and divide, the inverse y transform;
 //   k_mm_inv_xt : the inverse time DCT of every column, the inverse x transform -> phi.
-// At 180x135x3, P = 24 (events, one GB300): 36, 40 and 27 us against 138, 185 and 234 us of the dense sums; the
-// iteration 117 against 575 us.  What bounds them there is latency at three blocks per SM (issue slots 39-56 % busy,
+// At 180x135x3, P = 24 (events, one GB300): 35, 39 and 25 us against 138, 185 and 234 us of the dense sums; the
+// iteration 111 against 575 us.  What bounds them there is latency at three blocks per SM (issue slots 39-58 % busy,
 // 1.7 M cells leave 10 warps per SM with this register tile); the multiply-adds alone would take 5-8 us each.
 // They replace the dense sums of k_rhs_fwd_xt, k_solve_yc and k_inv_xt (one output and n dependent steps per
 // thread), which remain for planes that do not fit shared memory in this layout and for FP64 grids whose pipe they load
@@ -119,7 +119,7 @@ __device__ __forceinline__ void mm_zero(T (&acc)[RT][E]) {
 // Tables on their way through shared memory: chunks of kMmK rows in kMmStages slots.  The slots come first in a block's
 // shared memory, so that they start on lines of 128 bytes as the tables do in global memory: a warp's copy of 512 bytes
 // falls apart into more pieces otherwise (224x97x1, P = 16: y pass 15.8 us, 20.0 with the tables 16 bytes further, 21.7 with
-// the slots 48 bytes off; 180x135x3, P = 24 38.9, 42.5, 42.3).
+// the slots 48 bytes off; 180x135x3, P = 24 38.9, 42.5, 42.3, its L2 traffic 68 MB, 128 with the slots off).
 constexpr int kMmK = 8, kMmStages = 3;
 __host__ __device__ inline int mm_buf(int l0, int lf, int li) { return kMmStages * kMmK * (lf > 2 * li ? lf : 2 * li); }
 
